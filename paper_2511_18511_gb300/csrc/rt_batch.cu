@@ -174,9 +174,10 @@ __global__ void __launch_bounds__(BLOCK, MINB)
         const InstDesc& d = P.d[inst];
         const Geom& G = d.G;
         bool ended = false;
+        const bool sparse = sparse_warp();
 #pragma unroll 1
         for (int u = 0; u < STEPS; ++u)
-            if (trace_step(C, G, ts, sink)) {
+            if (trace_step(C, G, ts, sink, sparse)) {
                 ended = true;
                 break;
             }

@@ -71,6 +71,20 @@ __device__ __forceinline__ void node_vals(const double* __restrict__ c_mps, int 
     v[3] = 1.0 / c;
 }
 
+// Storage order of a cell's coefficients f[field][a, bx, by, bxy], fields (c, gx, gy, s).
+__device__ __forceinline__ void pack_cell(const double f[4][4], CellCoef<double>& o) {
+    o.c = D4{f[0][0], f[0][1], f[0][2], f[0][3]};
+    o.gx = D4{f[1][0], f[1][1], f[1][2], f[1][3]};
+    o.gy = D4{f[2][0], f[2][1], f[2][2], f[2][3]};
+    o.s = D4{f[3][0], f[3][1], f[3][2], f[3][3]};
+}
+__device__ __forceinline__ void pack_cell(const float f[4][4], CellCoef<float>& o) {
+    o.p.v[0] = make_float4(f[0][0], f[3][0], f[0][1], f[3][1]);
+    o.p.v[1] = make_float4(f[0][2], f[3][2], f[0][3], f[3][3]);
+    o.p.v[2] = make_float4(f[1][0], f[2][0], f[1][1], f[2][1]);
+    o.p.v[3] = make_float4(f[1][2], f[2][2], f[1][3], f[2][3]);
+}
+
 // A1: per-cell bilinear coefficients of the four nodal fields, computed in FP64
 // and stored in the marching precision; flags c <= 0 or NaN.
 template <typename T>
@@ -86,18 +100,15 @@ __global__ void k_pack(const double* __restrict__ c_mps, int nx, int ny, CellCoe
         const double cs[4] = {v00[0], v10[0], v01[0], v11[0]};
         for (int q = 0; q < 4; ++q)
             if (!(cs[q] > 0.0) || !isfinite(cs[q])) atomicOr(bad, 1);
-        typename Vec4T<T>::type f[4];
+        T f[4][4];   // per field: a, bx, by, bxy
         for (int q = 0; q < 4; ++q) {
-            f[q].x = (T)v00[q];
-            f[q].y = (T)(v10[q] - v00[q]);
-            f[q].z = (T)(v01[q] - v00[q]);
-            f[q].w = (T)((v11[q] - v10[q]) - (v01[q] - v00[q]));
+            f[q][0] = (T)v00[q];
+            f[q][1] = (T)(v10[q] - v00[q]);
+            f[q][2] = (T)(v01[q] - v00[q]);
+            f[q][3] = (T)((v11[q] - v10[q]) - (v01[q] - v00[q]));
         }
         CellCoef<T> o;
-        o.c = f[0];
-        o.gx = f[1];
-        o.gy = f[2];
-        o.s = f[3];
+        pack_cell(f, o);
         F[k] = o;
     }
 }
@@ -283,9 +294,10 @@ __global__ void __launch_bounds__(kLinkBlock, LinkBlocks<T, I, REC>::v) k_link(G
             active = true;
         }
         bool ended = false;
+        const bool sparse = sparse_warp();
 #pragma unroll 1
         for (int u = 0; u < kLinkSteps; ++u)
-            if (trace_step(C, G, ts, ns)) {
+            if (trace_step(C, G, ts, ns, sparse)) {
                 ended = true;
                 break;
             }

@@ -111,6 +111,42 @@ __device__ __forceinline__ float rcp_approx(float x) {
 }
 __device__ __forceinline__ double rcp_approx(double x) { return 1.0 / x; }
 
+// Two FP32 values in one 64-bit register pair. Each operation below is one
+// instruction that rounds both halves exactly as its scalar form does, so the
+// march's (x, y) pairs cost half the issue slots of scalar code.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 pk2(float x, float y) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ F2 dup2(float x) { return pk2(x, x); }
+__device__ __forceinline__ void unpk2(F2 a, float& x, float& y) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v));
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) {
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+
 // ---------------------------------------------------------------- field cache
 
 // The cell (i, j) and in-cell fractions (tx, ty) of a point given by fractions
@@ -178,6 +214,118 @@ struct Cell {
 
     // slowness at fractions (tx, ty) of the cached cell
     __device__ __forceinline__ T slow(T tx, T ty) const { return sa + tx * sbx + ty * (sby + tx * sbxy); }
+};
+
+// The FP32 cell: the same bilinear coefficients as two pairs of fields, (c, s)
+// and (h dc/dx, h dc/dy), so that a sample is packed arithmetic. o = (ci - pi,
+// cj - pj) of a step carries fractions of the step's own cell to the cached
+// one, which makes the in-cell test of a stage three instructions.
+struct __align__(32) CellPairs {
+    float4 v[4];   // (a_c, a_s, bx_c, bx_s), (by_c, by_s, bxy_c, bxy_s), then the same of (gx, gy)
+};
+
+template <>
+struct CellCoef<float> {
+    CellPairs p;
+};
+
+// The cell i of fraction u in [-1, 2) of cell c, and the offset c - i.
+__device__ __forceinline__ void axis_move(float u, int c, int& i, float& o) {
+    const bool lo = u < 0.0f, hi = u >= 1.0f;
+    o = lo ? 1.0f : (hi ? -1.0f : 0.0f);
+    i = c + (lo ? -1 : (hi ? 1 : 0));
+}
+
+template <>
+struct Cell<float> {
+    using V = CellCoef<float>;
+    const V* __restrict__ F;
+    int nx, ny;
+    int pi, pj;                       // cached cell
+    F2 sa, sx, sy, sxy;               // (c, s) = sa + tx sx + ty (sy + tx sxy)
+    F2 ga, gx, gy, gxy;               // (h dc/dx, h dc/dy)
+
+    __device__ __forceinline__ void load(int i, int j) {
+        pi = i;
+        pj = j;
+        // clamp for memory safety; rays stay inside by the ring/grid check
+        const unsigned w = (unsigned)(nx - 1);
+        const V* p = F + min((unsigned)j * w + (unsigned)i, w * (unsigned)(ny - 1) - 1u);
+        asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(sa.v), "=l"(sx.v), "=l"(sy.v), "=l"(sxy.v) : "l"(p));
+        asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4 + 32];" : "=l"(ga.v), "=l"(gx.v), "=l"(gy.v), "=l"(gxy.v) : "l"(p));
+    }
+
+    // Moves the cache to the cell of a point outside it: its fractions and the
+    // offset of the step's cell (ci, cj) from it.
+    __device__ __forceinline__ void move(int ci, int cj, float u, float v, float& ox, float& oy, float& tx, float& ty) {
+        int i, j;
+        axis_move(u, ci, i, ox);
+        axis_move(v, cj, j, oy);
+        if (!(u >= -1.0f && u < 2.0f && v >= -1.0f && v < 2.0f)) {   // steps longer than a cell
+            const float fu = floorf(u), fv = floorf(v);
+            i = ci + (int)fu;
+            j = cj + (int)fv;
+            ox = -fu;
+            oy = -fv;
+        }
+        tx = u + ox;
+        ty = v + oy;
+        load(i, j);
+    }
+
+    // First point of a step, (u, v) relative to cell (ci, cj).
+    __device__ __forceinline__ void seek(int ci, int cj, float u, float v, float& ox, float& oy, float& tx, float& ty) {
+        // opaque zeros: known ones would let the compiler clone the rest of the
+        // step for the unmoved case, which keeps the lanes of a warp apart
+        asm("mov.f32 %0, 0f00000000;" : "=f"(ox));
+        asm("mov.f32 %0, 0f00000000;" : "=f"(oy));
+        tx = u;
+        ty = v;
+        if (!(ci == pi && cj == pj && max(__float_as_uint(u), __float_as_uint(v)) < 0x3f800000u))
+            move(ci, cj, u, v, ox, oy, tx, ty);
+    }
+    // A later point of the step. Bits below those of 1.0f are the fractions in
+    // [0, 1): u + ox is then the fraction cell_locate gives for that cell.
+    __device__ __forceinline__ void next(int ci, int cj, F2 p, float& ox, float& oy, float& tx, float& ty) {
+        unpk2(add2(p, pk2(ox, oy)), tx, ty);
+        if (max(__float_as_uint(tx), __float_as_uint(ty)) >= 0x3f800000u) {
+            float u, v;
+            unpk2(p, u, v);
+            move(ci, cj, u, v, ox, oy, tx, ty);
+        }
+    }
+    __device__ __forceinline__ F2 cs(float tx, float ty) const {
+        const F2 x = dup2(tx);
+        return fma2(dup2(ty), fma2(x, sxy, sy), fma2(x, sx, sa));
+    }
+    __device__ __forceinline__ float c(float tx, float ty) const {
+        float a, b, d, e, t;
+        unpk2(sa, a, t);
+        unpk2(sx, b, t);
+        unpk2(sy, d, t);
+        unpk2(sxy, e, t);
+        return fmaf(ty, fmaf(tx, e, d), fmaf(tx, b, a));
+    }
+    __device__ __forceinline__ F2 grad(float tx, float ty) const {
+        const F2 x = dup2(tx);
+        return fma2(dup2(ty), fma2(x, gxy, gy), fma2(x, gx, ga));
+    }
+
+    __device__ __forceinline__ void at(int ci, int cj, float u, float v, float& c_, float& gx_, float& gy_, float& tx,
+                                       float& ty) {
+        float ox, oy;
+        seek(ci, cj, u, v, ox, oy, tx, ty);
+        c_ = c(tx, ty);
+        unpk2(grad(tx, ty), gx_, gy_);
+    }
+    __device__ __forceinline__ float slow(float tx, float ty) const {
+        float a, b, d, e, t;
+        unpk2(sa, t, a);
+        unpk2(sx, t, b);
+        unpk2(sy, t, d);
+        unpk2(sxy, t, e);
+        return fmaf(ty, fmaf(tx, e, d), fmaf(tx, b, a));
+    }
 };
 
 // ---------------------------------------------------------------- direction
@@ -345,12 +493,208 @@ __device__ __forceinline__ void heun_step(CellT& C, const RayState<T>& S, T H, R
     N.fy = nfy;
 }
 
+// ((g.e) e - g) / c of the FP32 march, in the operation order of ray_rhs with
+// the signs of both factors flipped (exact).
+__device__ __forceinline__ F2 ray_rhs2(float c, F2 g, F2 e) {
+    float gx, gy, ex, ey;
+    unpk2(g, gx, gy);
+    unpk2(e, ex, ey);
+    const float nic = rcp_approx(-c);
+    const float ngd = fmaf(-gy, ey, -__fmul_rn(gx, ex));
+    return mul2(fma2(dup2(ngd), e, g), dup2(nic));
+}
+// a + the same, the product with 1/c rounded once with the sum
+__device__ __forceinline__ F2 add_rhs2(F2 a, float c, F2 g, F2 e) {
+    float gx, gy, ex, ey;
+    unpk2(g, gx, gy);
+    unpk2(e, ex, ey);
+    const float nic = rcp_approx(-c);
+    const float ngd = fmaf(-gy, ey, -__fmul_rn(gx, ex));
+    return fma2(fma2(dup2(ngd), e, g), dup2(nic), a);
+}
+
+// Position and direction of a step from its increments: position by sum Hp
+// E + H d_lo, direction by Hp K, both as rk4_step forms them.
+__device__ __forceinline__ void commit2(const RayState<float>& S, float H, float Hp, F2 E, F2 K, RayState<float>& N) {
+    const F2 dl = pk2(S.d.ex, S.d.ey), hp = dup2(Hp), h1 = dup2(H);
+    // compensated position
+    const F2 f = pk2(S.fx, S.fy), l = pk2(S.lx, S.ly);
+    const F2 inc = fma2(h1, dl, mul2(hp, E));
+    const F2 s = add2(f, inc), b = sub2(s, f);
+    F2 lo = add2(l, add2(sub2(f, sub2(s, b)), sub2(inc, b)));
+    const F2 nf = add2(s, lo);
+    lo = sub2(lo, sub2(nf, s));
+    unpk2(lo, N.lx, N.ly);
+    // compensated direction, renormalised
+    const F2 d = pk2(S.d.x, S.d.y);
+    const F2 x = fma2(hp, K, d), nb = sub2(d, x);
+    F2 e = add2(dl, add2(sub2(d, add2(x, nb)), fma2(hp, K, nb)));
+    float dx, dy, ex, ey;
+    unpk2(x, dx, dy);
+    unpk2(e, ex, ey);
+    const float q = fmaf(dx, ex, __fmul_rn(dy, ey));
+    const float er = fmaf(2.0f, q, fmaf(dx, dx, fmaf(dy, dy, -1.0f)));
+    const F2 delta = dup2(__fmul_rn(er, fmaf(0.375f, er, -0.5f)));
+    e = fma2(add2(x, e), delta, e);
+    const F2 xs = add2(x, e);
+    e = sub2(e, sub2(xs, x));
+    unpk2(xs, N.d.x, N.d.y);
+    unpk2(e, N.d.ex, N.d.ey);
+    float nfx, nfy;
+    unpk2(nf, nfx, nfy);
+    N.ci = S.ci;
+    N.cj = S.cj;
+    // into the next cell: f - 1 is exact for f in [1, 2); f + 1 for f < 0 rounds,
+    // so it goes through the residual (both axes at once, add_frac's operations)
+    if (max(__float_as_uint(nfx), __float_as_uint(nfy)) >= 0x3f800000u) {
+        const bool xl = nfx < 0.0f, xh = nfx >= 1.0f, yl = nfy < 0.0f, yh = nfy >= 1.0f;
+        const F2 a = pk2(xl ? 1.0f : (xh ? -1.0f : 0.0f), yl ? 1.0f : (yh ? -1.0f : 0.0f));
+        const F2 t = add2(nf, a), tb = sub2(t, nf);
+        F2 r = add2(lo, add2(sub2(nf, sub2(t, tb)), sub2(a, tb)));
+        const F2 t2 = add2(t, r);
+        r = sub2(r, sub2(t2, t));
+        float x1, y1, x2, y2, rx, ry;
+        unpk2(t, x1, y1);
+        unpk2(t2, x2, y2);
+        unpk2(r, rx, ry);
+        nfx = xl ? x2 : x1;
+        nfy = yl ? y2 : y1;
+        if (xl) N.lx = rx;
+        if (yl) N.ly = ry;
+        N.ci += xl ? -1 : (xh ? 1 : 0);
+        N.cj += yl ? -1 : (yh ? 1 : 0);
+    }
+    N.fx = nfx;
+    N.fy = nfy;
+}
+
+// rk4_step of the FP32 bilinear march: the same operations on packed pairs,
+// bit for bit. The march issues instructions (a full GPU) or waits for its own
+// dependent chain (few rays); it moves almost no memory. Packing takes a lone
+// ray from 258 to 186 instructions a step; a packed operation has a longer
+// latency, so that alone saved 4 % of a full launch and nothing of a lone ray.
+// The rest came from what surrounds the arithmetic: a cell move of 20
+// instructions in place of 45 (every lane that leaves its cell costs the whole
+// warp one), two 32-byte loads a cell, one branch for the wrap of both axes,
+// one for all rare ends of a step. Each stage's cell lookup comes before the
+// slopes of the stage before it, so that those slopes and the new sample are
+// one block of independent work. Together, on the breast medium (1024^2, 512
+// transducers): recording link 56 -> 45.5 ms cold, 25.3 -> 22.2 ms warm; plain
+// link 50 -> 40.4 and 19.3 -> 15.9 ms; adjoint 24.1 -> 20.8 ms; one ray 345 ->
+// 266 ns a step. Loading the next cell ahead of its use (L1 prefetch, cp.async
+// or a plain load at the entry of a cell) and scalar slopes were no faster.
+__device__ __forceinline__ void rk4_slopes(Cell<float>& C, const RayState<float>& S, float H, F2& E, F2& K,
+                                           float& s_here, float& tx1, float& ty1, int& i1, int& j1) {
+    const F2 hh = dup2(0.5f * H), h1 = dup2(H), f = pk2(S.fx, S.fy), d = pk2(S.d.x, S.d.y), two = dup2(2.0f);
+    float ox, oy, tx, ty, c;
+    C.seek(S.ci, S.cj, S.fx, S.fy, ox, oy, tx1, ty1);
+    i1 = C.pi;
+    j1 = C.pj;
+    unpk2(C.cs(tx1, ty1), c, s_here);
+    F2 g = C.grad(tx1, ty1);
+    C.next(S.ci, S.cj, fma2(hh, d, f), ox, oy, tx, ty);
+    const F2 k1 = ray_rhs2(c, g, d);
+    c = C.c(tx, ty);
+    g = C.grad(tx, ty);
+    const F2 e2 = fma2(hh, k1, d);
+    C.next(S.ci, S.cj, fma2(hh, e2, f), ox, oy, tx, ty);
+    const F2 k2 = ray_rhs2(c, g, e2);
+    c = C.c(tx, ty);
+    g = C.grad(tx, ty);
+    const F2 e3 = fma2(hh, k2, d);
+    C.next(S.ci, S.cj, fma2(h1, e3, f), ox, oy, tx, ty);
+    const F2 k3 = ray_rhs2(c, g, e3);
+    const F2 e4 = fma2(h1, k3, d);
+    c = C.c(tx, ty);
+    g = C.grad(tx, ty);
+    E = add2(fma2(two, add2(e2, e3), d), e4);
+    K = add_rhs2(fma2(two, add2(k2, k3), k1), c, g, e4);
+}
+
+// The same for a step whose four samples all lie in the cached cell, assumed
+// first and tested last: one branch a step, and the samples' arithmetic
+// overlaps. Returns whether they did; if not, the outputs mean nothing.
+__device__ __forceinline__ bool rk4_slopes_inside(const Cell<float>& C, const RayState<float>& S, float H, F2& E, F2& K,
+                                                  float& s_here) {
+    const F2 hh = dup2(0.5f * H), h1 = dup2(H), f = pk2(S.fx, S.fy), d = pk2(S.d.x, S.d.y), two = dup2(2.0f);
+    float x, y, c;
+    unsigned m = max(__float_as_uint(S.fx), __float_as_uint(S.fy));
+    unpk2(fma2(hh, d, f), x, y);
+    m = max(m, max(__float_as_uint(x), __float_as_uint(y)));
+    const float c2 = C.c(x, y);
+    const F2 g2 = C.grad(x, y);
+    unpk2(C.cs(S.fx, S.fy), c, s_here);
+    const F2 k1 = ray_rhs2(c, C.grad(S.fx, S.fy), d);
+    const F2 e2 = fma2(hh, k1, d);
+    unpk2(fma2(hh, e2, f), x, y);
+    m = max(m, max(__float_as_uint(x), __float_as_uint(y)));
+    const F2 k2 = ray_rhs2(c2, g2, e2);
+    const F2 e3 = fma2(hh, k2, d);
+    const F2 k3 = ray_rhs2(C.c(x, y), C.grad(x, y), e3);
+    unpk2(fma2(h1, e3, f), x, y);
+    m = max(m, max(__float_as_uint(x), __float_as_uint(y)));
+    const F2 e4 = fma2(h1, k3, d);
+    E = add2(fma2(two, add2(e2, e3), d), e4);
+    K = add_rhs2(fma2(two, add2(k2, k3), k1), C.c(x, y), C.grad(x, y), e4);
+    return S.ci == C.pi && S.cj == C.pj && m < 0x3f800000u;
+}
+
+__device__ __forceinline__ void rk4_step(Cell<float>& C, const RayState<float>& S, float H, RayState<float>& N,
+                                         float& s_here, float& tx1, float& ty1, int& i1, int& j1, bool sparse) {
+    F2 E, K;
+    bool inside = false;
+    if (sparse) {
+        tx1 = S.fx;
+        ty1 = S.fy;
+        i1 = S.ci;
+        j1 = S.cj;
+        inside = rk4_slopes_inside(C, S, H, E, K, s_here);
+    }
+    if (!inside) rk4_slopes(C, S, H, E, K, s_here, tx1, ty1, i1, j1);
+    commit2(S, H, H / 6.0f, E, K, N);
+}
+
+// heun_step of the FP32 bilinear march, packed likewise.
+__device__ __forceinline__ void heun_step(Cell<float>& C, const RayState<float>& S, float H, RayState<float>& N,
+                                          float& s_here, float& tx1, float& ty1, int& i1, int& j1) {
+    const float Hh = 0.5f * H;
+    const F2 h1 = dup2(H), f = pk2(S.fx, S.fy), d = pk2(S.d.x, S.d.y);
+    float ox, oy, tx, ty, c;
+    C.seek(S.ci, S.cj, S.fx, S.fy, ox, oy, tx1, ty1);
+    i1 = C.pi;
+    j1 = C.pj;
+    unpk2(C.cs(tx1, ty1), c, s_here);
+    F2 g = C.grad(tx1, ty1);
+    C.next(S.ci, S.cj, fma2(h1, d, f), ox, oy, tx, ty);
+    const F2 k1 = ray_rhs2(c, g, d);
+    const F2 e2 = fma2(h1, k1, d);
+    c = C.c(tx, ty);
+    g = C.grad(tx, ty);
+    const F2 K = add_rhs2(k1, c, g, e2);
+    commit2(S, H, Hh, add2(d, e2), K, N);
+}
+
+// Lanes of a warp up to which a step is first tried inside the cached cell.
+// Each ray leaves its cell about every eighth step, and the warp then pays for
+// both forms of the step: worth it for one to three lanes (one ray 300 ns a
+// step against 348 without at the time; 1 or 6 lanes in place of 3 change the
+// cold link by less than its runs differ). One-trace kernels of wide warps
+// leave the form out: it made the adjoint 10 % slower through its registers.
+constexpr int kSparseLanes = 3;
+__device__ __forceinline__ bool sparse_warp() { return __popc(__activemask()) <= kSparseLanes; }
+
 // The step of the configured integrator (uniform over a launch).
 template <typename T, typename CellT>
 __device__ __forceinline__ void ray_step(CellT& C, const Geom& G, const RayState<T>& S, T H, RayState<T>& N,
-                                         T& s_here, T& tx1, T& ty1, int& i1, int& j1) {
+                                         T& s_here, T& tx1, T& ty1, int& i1, int& j1, bool) {
     if (G.heun) heun_step(C, S, H, N, s_here, tx1, ty1, i1, j1);
     else rk4_step(C, S, H, N, s_here, tx1, ty1, i1, j1);
+}
+__device__ __forceinline__ void ray_step(Cell<float>& C, const Geom& G, const RayState<float>& S, float H,
+                                         RayState<float>& N, float& s_here, float& tx1, float& ty1, int& i1, int& j1,
+                                         bool sparse) {
+    if (G.heun) heun_step(C, S, H, N, s_here, tx1, ty1, i1, j1);
+    else rk4_step(C, S, H, N, s_here, tx1, ty1, i1, j1, sparse);
 }
 
 // |x|^2 - (R/h)^2 in cell^2 units, exact integer part plus a small fractional
@@ -431,7 +775,6 @@ struct TraceState {
     int flags;                // bit0 step cap, bit1 left outward at once
     int iL, jL;               // cell and fractions of the last full-step point
     T txL, tyL;
-    int steps;                // RK4 steps of this trace (incl. landing)
 };
 
 // Starts a trace at (xe, ye) with unit launch direction (c, s).
@@ -454,7 +797,6 @@ __device__ __forceinline__ void trace_begin_cs(TraceState<T>& ts, const Geom& G,
     ts.flags = 0;
     ts.iL = ts.jL = 0;
     ts.txL = ts.tyL = (T)0;
-    ts.steps = 0;
 }
 
 template <typename T>
@@ -468,51 +810,55 @@ __device__ __forceinline__ void trace_begin(TraceState<T>& ts, const Geom& G, do
 // outside the ring (flags bit1 if that was the very first step) or the step
 // cap was reached (flags bit0). On exit ts.S is still the last inside point.
 template <typename T, typename CellT, typename Sink>
-__device__ __forceinline__ bool trace_step(CellT& C, const Geom& G, TraceState<T>& ts, Sink& sink) {
-    if (ts.m >= G.max_steps_i) {
-        ts.flags |= 1;
-        return true;
-    }
+__device__ __forceinline__ bool trace_step(CellT& C, const Geom& G, TraceState<T>& ts, Sink& sink, bool sparse) {
     const T H = StepK<T>::H(G);
-    const T dsT = StepK<T>::ds(G);
+    T w = StepK<T>::ds(G);
     RayState<T> N;
     T tx1, ty1;
     int i1, j1;
-    ray_step(C, G, ts.S, H, N, ts.s_cur, tx1, ty1, i1, j1);
-    ++ts.steps;
-    bool ends_out = false;
+    ray_step(C, G, ts.S, H, N, ts.s_cur, tx1, ty1, i1, j1, sparse);
+    int end = 0;   // 1: the step ended on or outside the ring, 2: as the first step, 3: the step cap
+    // Everything that can only happen on a step that may reach the ring, on the
+    // first step (safe starts at 0) or at the step cap is behind this one test.
     if (--ts.safe < 0) {
         const T ex = ring_excess(G, N);
-        ends_out = ex >= (T)0;
-        if (!ends_out) {
+        if (ex >= (T)0) end = ts.m == 0 ? 2 : 1;
+        if (ts.m == 0) {
+            ts.s_first = ts.s_cur;
+            ts.Scomp = ts.s_cur;   // the sum below stays 0 on this step
+            w *= (T)0.5;
+        }
+        if (!end) {
             // distance to the ring in cells, -ex / (R + r); no step moves farther than ~H
             const T Rc = StepK<T>::Rc(G);
             const T r = sqrt(Rc * Rc + ex);
             const T dist = -ex / (Rc + r);
-            ts.safe = (int)(dist * (T)0.98 / H) - 1;
+            const int left = G.max_steps_i - 2 - ts.m;   // free steps before the last one allowed
+            ts.safe = min((int)(dist * (T)0.98 / H) - 1, left);
+            if (left < 0) end = 3;
         }
     }
-    if (ts.m == 0) {
-        if (ends_out) {   // left outward: no path, no weights
-            ts.flags |= 2;
-            return true;
-        }
-        ts.s_first = ts.s_cur;
-        sink.add(i1, j1, tx1, ty1, (T)0.5 * dsT);
-    } else {
-        const T y = ts.s_cur - ts.Scomp;
-        const T t = ts.Ssum + y;
-        ts.Scomp = (t - ts.Ssum) - y;
-        ts.Ssum = t;
-        sink.add(i1, j1, tx1, ty1, dsT);
-        if (ends_out) {
-            ts.iL = i1; ts.jL = j1; ts.txL = tx1; ts.tyL = ty1;
-            return true;
-        }
+    // opaque: with the end codes known per path the compiler clones the rest of
+    // the step, and the lanes of a warp that took this branch stay apart
+    asm volatile("" : "+r"(end));
+    if (end == 2) {   // left outward: no path, no weights
+        ts.s_first = (T)0;
+        ts.flags |= 2;
+        return true;
+    }
+    const T y = ts.s_cur - ts.Scomp;
+    const T t = ts.Ssum + y;
+    ts.Scomp = (t - ts.Ssum) - y;
+    ts.Ssum = t;
+    sink.add(i1, j1, tx1, ty1, w);
+    if (end == 1) {
+        ts.iL = i1; ts.jL = j1; ts.txL = tx1; ts.tyL = ty1;
+        return true;
     }
     ts.S = N;
     ++ts.m;
-    return false;
+    if (end == 3) ts.flags |= 1;
+    return end != 0;
 }
 
 // Landing, travel time and final weights of an ended trace. The endpoint
@@ -526,7 +872,7 @@ __device__ TraceOut trace_end(CellT& C, const Geom& G, TraceState<T>& ts, double
         // step cap: no interception; report the current point
         abs_pos(G, ts.S, out.hx, out.hy);
         out.T = G.ds * (0.5 * (double)ts.s_first + ((double)ts.Ssum - (double)ts.Scomp));
-        out.steps = ts.steps;
+        out.steps = ts.m;
         sink.finish();
         return out;
     }
@@ -534,7 +880,7 @@ __device__ TraceOut trace_end(CellT& C, const Geom& G, TraceState<T>& ts, double
         out.T = 0.0;
         out.hx = xe;
         out.hy = ye;
-        out.steps = ts.steps;
+        out.steps = 1;
         sink.finish();
         return out;
     }
@@ -553,8 +899,7 @@ __device__ TraceOut trace_end(CellT& C, const Geom& G, TraceState<T>& ts, double
     T s_dummy, txd, tyd;
     int id, jd;
     for (int it = 0; it < 2; ++it) {
-        ray_step(C, G, S, (T)(t / G.h), N, s_dummy, txd, tyd, id, jd);
-        ++ts.steps;
+        ray_step(C, G, S, (T)(t / G.h), N, s_dummy, txd, tyd, id, jd, false);
         double NX, NY;
         abs_pos(G, N, NX, NY);
         double r = sqrt(NX * NX + NY * NY);
@@ -563,8 +908,7 @@ __device__ TraceOut trace_end(CellT& C, const Geom& G, TraceState<T>& ts, double
         if (!(t >= 0)) t = 0;
         if (t > G.ds) t = G.ds;
     }
-    ray_step(C, G, S, (T)(t / G.h), N, s_dummy, txd, tyd, id, jd);
-    ++ts.steps;
+    ray_step(C, G, S, (T)(t / G.h), N, s_dummy, txd, tyd, id, jd, false);
     double MX, MY;
     abs_pos(G, N, MX, MY);
     T c_, gx_, gy_, txM, tyM;
@@ -577,7 +921,7 @@ __device__ TraceOut trace_end(CellT& C, const Geom& G, TraceState<T>& ts, double
     out.T = G.ds * (0.5 * (double)ts.s_first + S_int - 0.5 * sL) + 0.5 * t * (sL + sM) + sM * corr;
     out.hx = MX;
     out.hy = MY;
-    out.steps = ts.steps;
+    out.steps = ts.m + 4;   // the full steps inside, the one that crossed, three to land
     // alpha_{M-1} = (ds + ds')/2 (ds was given by trace_step), alpha_M = ds'/2 + corr
     sink.add(ts.iL, ts.jL, ts.txL, ts.tyL, (T)(0.5 * (t - G.ds)));
     sink.add(iM, jM, txM, tyM, (T)(0.5 * t + corr));
@@ -590,10 +934,10 @@ __device__ TraceOut trace_end(CellT& C, const Geom& G, TraceState<T>& ts, double
 // endpoint weight) with its cell and fractions.
 template <typename T, typename CellT, typename Sink>
 __device__ TraceOut trace_ray(CellT& C, const Geom& G, double xe, double ye, double theta, double xr,
-                              double yr, Sink& sink) {
+                              double yr, Sink& sink, bool sparse = false) {
     TraceState<T> ts;
     trace_begin(ts, G, xe, ye, theta);
-    while (!trace_step(C, G, ts, sink)) {
+    while (!trace_step(C, G, ts, sink, sparse)) {
     }
     return trace_end(C, G, ts, xe, ye, xr, yr, sink);
 }
