@@ -565,6 +565,13 @@ struct RecSink {
     }
 };
 
+// One-trace-per-ray launches (blocks of 128): only the first `lanes` lanes of
+// each warp take a ray, so that few rays run in many warps of few lanes.
+struct Spread {
+    int lanes, blocks;
+};
+Spread spread_for(long long n, int prec);
+
 // Recording target of a linking launch (rt_link_rows); runs == null: none.
 struct RowRec {
     rt_run* runs;

@@ -23,6 +23,50 @@ constexpr int kBlock = 128;
 
 static int grid_for(int n) { return (n + kBlock - 1) / kBlock; }
 
+// SMs of the current device (cached per device).
+static int sm_count() {
+    static std::atomic<int> cache[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) dev = 0;
+    int v = cache[dev].load(std::memory_order_relaxed);
+    if (!v) {
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        if (v <= 0) v = 152;
+        cache[dev].store(v, std::memory_order_relaxed);
+    }
+    return v;
+}
+
+// Warps per SM that few rays are spread over. A march is bound by the latency
+// of its own chain as long as a scheduler has two or three warps, and a warp
+// steps faster the fewer lanes it has (266 ns a step with one, 890 with 32:
+// every lane that leaves its cell costs the warp a reload), so rays go to more
+// warps first. Beyond about four warps a scheduler the warps' instructions
+// queue and fuller warps are better: 63 rays of a 128^2 grid 1.10 -> 0.38 ms
+// (two warps -> 63), linking 4,032 pairs 1.58 ms at 16 warps an SM and 1.42 at
+// 8 (all 24 resident: 1.63), 65,280 pairs 15.0 and 14.9 ms (15.8); the one-trace
+// launches measure alike from 8 to 16, 12 a little better at 65,280 rays.
+constexpr int kSpreadWarps = 12, kLinkSpreadWarps = 8;
+// FP64 goes the other way: its instructions occupy the pipe per group of lanes
+// whether or not all of them are at work. 4,032 pairs linked and scattered on a
+// 128^2 grid: 29.7 ms at 3 lanes a warp, 20.6 at 8, 22.0 at 32; one-trace
+// launches keep full warps (20.6 against 21.8 ms at 8).
+constexpr int kMinLanes64 = 8;
+
+Spread spread_for(long long n, int prec) {
+    if (prec == RT_FP64) return Spread{32, (int)((n + kBlock - 1) / kBlock)};
+    const long long warps = (long long)sm_count() * kSpreadWarps;
+    const long long lanes = std::min<long long>(32, std::max<long long>(1, (n + warps - 1) / warps));
+    const long long per_block = lanes * (kBlock / 32);
+    return Spread{(int)lanes, (int)((n + per_block - 1) / per_block)};
+}
+// The ray of a thread of such a launch, INT_MAX for an idle lane.
+__device__ __forceinline__ int spread_slot(int lanes) {
+    const int lane = threadIdx.x & 31;
+    return lane < lanes ? (int)((blockIdx.x * (unsigned)kBlock + threadIdx.x) >> 5) * lanes + lane : INT_MAX;
+}
+
 size_t node_bytes(int prec, int interp) {
     if (interp == RT_BSPLINE) return prec == RT_FP64 ? sizeof(CellBS<double>) : sizeof(CellBS<float>);
     return prec == RT_FP64 ? sizeof(CellCoef<double>) : sizeof(CellCoef<float>);
@@ -163,30 +207,39 @@ __global__ void k_fan_mark(Geom G, const double* __restrict__ theta, int* need) 
 // G carries the fan's tracing step; margin (ds/R of the linking step) fixes
 // the fan's launch angles, which the linking predictions assume.
 template <typename T, int I>
-__global__ void __launch_bounds__(kBlock) k_fan(Geom G, const typename Samp<T, I>::Field* __restrict__ F, int K,
-                                                double margin, const int* __restrict__ need, double* fan,
-                                                unsigned long long* counters) {
-    const int id = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ long long fan_ray(const Geom& G, const typename Samp<T, I>::Field* __restrict__ F, int K,
+                                             double margin, const int* __restrict__ need, double* fan, int id) {
     const int rank = id / G.n_tx, e = id - rank * G.n_tx;
     const int half = K / 2;
     const int k = (rank & 1) ? half - (rank + 1) / 2 : half + rank / 2;
-    long long steps = 0;
-    if (id < G.n_tx * K && need[e] && !*G.bad_field) {
-        const double xe = G.tx[2 * e], ye = G.tx[2 * e + 1];
-        const double phi_e = atan2(ye, xe);
-        const double a_min = phi_e + 0.5 * kPi + margin, a_max = phi_e + 1.5 * kPi - margin;
-        const double step = (a_max - a_min) / (K - 1);
-        auto C = make_cell<T, I>(G, F);
-        NoSink ns;
-        const TraceOut o = trace_ray<T>(C, G, xe, ye, fan_theta(a_min, step, k), xe, ye, ns);
-        fan[(size_t)e * K + k] = (o.flags & 3) ? nan("") : mod_2pi(atan2(o.hy, o.hx) - phi_e);
-        steps = o.steps;
-    }
-    // every thread of the block reaches this point
+    if (!need[e] || *G.bad_field) return 0;
+    const double xe = G.tx[2 * e], ye = G.tx[2 * e + 1];
+    const double phi_e = atan2(ye, xe);
+    const double a_min = phi_e + 0.5 * kPi + margin, a_max = phi_e + 1.5 * kPi - margin;
+    const double step = (a_max - a_min) / (K - 1);
+    auto C = make_cell<T, I>(G, F);
+    NoSink ns;
+    const TraceOut o = trace_ray<T>(C, G, xe, ye, fan_theta(a_min, step, k), xe, ye, ns);
+    fan[(size_t)e * K + k] = (o.flags & 3) ? nan("") : mod_2pi(atan2(o.hy, o.hx) - phi_e);
+    return o.steps;
+}
+
+// Adds the warp's steps to counters[7]; every thread of the block gets here.
+__device__ __forceinline__ void count_steps(long long steps, unsigned long long* counters) {
     __syncwarp();
     unsigned long long v = (unsigned long long)steps;
     for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
     if ((threadIdx.x & 31) == 0 && v) atomicAdd(&counters[7], v);
+}
+
+template <typename T, int I>
+__global__ void __launch_bounds__(kBlock) k_fan(Geom G, const typename Samp<T, I>::Field* __restrict__ F, int K,
+                                                double margin, const int* __restrict__ need, double* fan,
+                                                unsigned long long* counters, int lanes) {
+    const int id = spread_slot(lanes);
+    long long steps = 0;
+    if (id < G.n_tx * K) steps = fan_ray<T, I>(G, F, K, margin, need, fan, id);
+    count_steps(steps, counters);
 }
 
 // Persistent linking kernel: each lane takes pairs from the queue, advances
@@ -364,8 +417,9 @@ template <typename T, int I>
 static void fan_impl(const Geom& G, const void* field, int fan_rays, double margin, double* fan,
                      const int* fan_need, unsigned long long* counters, cudaStream_t s) {
     const int nf = G.n_tx * fan_rays;
-    k_fan<T, I><<<grid_for(nf), kBlock, 0, s>>>(G, (const typename Samp<T, I>::Field*)field, fan_rays, margin,
-                                                fan_need, fan, counters);
+    const Spread sp = spread_for(nf, sizeof(T) == 8 ? RT_FP64 : RT_FP32_COMP);
+    k_fan<T, I><<<sp.blocks, kBlock, 0, s>>>(G, (const typename Samp<T, I>::Field*)field, fan_rays, margin, fan_need,
+                                             fan, counters, sp.lanes);
 }
 
 Geom with_step(const Geom& G, double ds) {
@@ -378,14 +432,23 @@ Geom with_step(const Geom& G, double ds) {
     return F;
 }
 
-cudaError_t launch_fan(const Geom& G, double fan_ds, const void* field, int prec, int fan_rays, const double* theta,
-                       double* fan, int* fan_need, unsigned long long* counters, cudaStream_t s) {
-    if (G.n_pairs == 0 || fan_rays < 2) return cudaSuccess;
+static double fan_margin(const Geom& G) { return fmax(G.ds / G.R, 1e-9); }
+
+// need[e] = 1 for the emitters of pairs that start cold.
+static cudaError_t mark_fans(const Geom& G, const double* theta, int* fan_need, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(fan_need, 0, sizeof(int) * (size_t)G.n_tx, s);
     if (e != cudaSuccess) return e;
     k_fan_mark<<<grid_for(G.n_pairs), kBlock, 0, s>>>(G, theta, fan_need);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fan(const Geom& G, double fan_ds, const void* field, int prec, int fan_rays, const double* theta,
+                       double* fan, int* fan_need, unsigned long long* counters, cudaStream_t s) {
+    if (G.n_pairs == 0 || fan_rays < 2) return cudaSuccess;
+    const cudaError_t e = mark_fans(G, theta, fan_need, s);
+    if (e != cudaSuccess) return e;
     const Geom F = fan_ds > 0.0 ? with_step(G, fan_ds) : G;
-    const double margin = fmax(G.ds / G.R, 1e-9);
+    const double margin = fan_margin(G);
     const bool bs = G.interp == RT_BSPLINE;
     if (prec == RT_FP64) {
         if (bs) fan_impl<double, RT_BSPLINE>(F, field, fan_rays, margin, fan, fan_need, counters, s);
@@ -402,14 +465,14 @@ static void link_impl(const Geom& G, const void* field, double tol, int max_iter
                       double* hit, int32_t* status, int32_t* iters, unsigned long long* counters, int* queue,
                       int fan_rays, double* fan, int slot, cudaStream_t s, const RowRec& rec = RowRec{},
                       const LinkRound& rd = LinkRound{}) {
-    // With fewer pairs than the persistent grid has lanes, the pairs are
-    // spread over all of its warps, ceil(pairs / warps) lanes each, rather
+    // With fewer pairs than kLinkSpreadWarps full warps per SM, the pairs are
+    // spread over that many warps, ceil(pairs / warps) lanes each, rather
     // than packed 32 to a warp on a few SMs (the linking is per pair, so the
     // results do not depend on the lanes that run them).
     const int pb = persistent_blocks(k_link<T, I, REC, ROUNDS>, slot);
-    const long long warps = (long long)pb * (kLinkBlock / 32);
+    const long long warps = std::min<long long>((long long)pb * (kLinkBlock / 32), (long long)sm_count() * kLinkSpreadWarps);
     const long long pairs = G.n_pairs;   // an upper bound of the pairs a rounds launch resumes
-    const int lanes = (int)std::min<long long>(32, std::max<long long>(1, (pairs + warps - 1) / warps));
+    const int lanes = (int)std::min<long long>(32, std::max<long long>(sizeof(T) == 8 ? kMinLanes64 : 1, (pairs + warps - 1) / warps));
     const long long per_block = (long long)lanes * (kLinkBlock / 32);
     const int nb = (int)std::min<long long>(pb, (pairs + per_block - 1) / per_block);
     k_link<T, I, REC, ROUNDS><<<nb, kLinkBlock, 0, s>>>(G, (const typename Samp<T, I>::Field*)field, tol, max_iter,
@@ -518,9 +581,10 @@ cudaError_t launch_link(const Geom& G, const void* field, int prec, double tol, 
 
 template <typename T, int I>
 __global__ void __launch_bounds__(kBlock) k_tof(Geom G, const typename Samp<T, I>::Field* __restrict__ F,
-                                                const double* theta, double* tof, double* hit) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= G.n_pairs) return;
+                                                const double* theta, double* tof, double* hit, int lanes) {
+    const int slot = spread_slot(lanes);
+    if (slot >= G.n_pairs) return;
+    const int k = queue_pair(G, slot);
     LinkCtx L;
     if (!setup_pair(G, k, L)) {
         tof[k] = nan("");
@@ -529,7 +593,7 @@ __global__ void __launch_bounds__(kBlock) k_tof(Geom G, const typename Samp<T, I
     }
     auto C = make_cell<T, I>(G, F);
     NoSink ns;
-    TraceOut o = trace_ray<T>(C, G, L.xe, L.ye, theta[k], L.xr, L.yr, ns);
+    TraceOut o = trace_ray<T>(C, G, L.xe, L.ye, theta[k], L.xr, L.yr, ns, lanes <= kSparseLanes);
     tof[k] = o.T;
     if (hit) { hit[2 * k] = o.hx; hit[2 * k + 1] = o.hy; }
 }
@@ -537,14 +601,15 @@ __global__ void __launch_bounds__(kBlock) k_tof(Geom G, const typename Samp<T, I
 cudaError_t launch_tof(const Geom& G, const void* field, int prec, const double* theta, double* tof,
                        double* hit, cudaStream_t s) {
     if (G.n_pairs == 0) return cudaSuccess;
-    const int nb = grid_for(G.n_pairs);
+    const Spread sp = spread_for(G.n_pairs, prec);
+    const int nb = sp.blocks;
     const bool bs = G.interp == RT_BSPLINE;
     if (prec == RT_FP64) {
-        if (bs) k_tof<double, RT_BSPLINE><<<nb, kBlock, 0, s>>>(G, (const CellBS<double>*)field, theta, tof, hit);
-        else k_tof<double, RT_BILINEAR><<<nb, kBlock, 0, s>>>(G, (const CellCoef<double>*)field, theta, tof, hit);
+        if (bs) k_tof<double, RT_BSPLINE><<<nb, kBlock, 0, s>>>(G, (const CellBS<double>*)field, theta, tof, hit, sp.lanes);
+        else k_tof<double, RT_BILINEAR><<<nb, kBlock, 0, s>>>(G, (const CellCoef<double>*)field, theta, tof, hit, sp.lanes);
     } else {
-        if (bs) k_tof<float, RT_BSPLINE><<<nb, kBlock, 0, s>>>(G, (const CellBS<float>*)field, theta, tof, hit);
-        else k_tof<float, RT_BILINEAR><<<nb, kBlock, 0, s>>>(G, (const CellCoef<float>*)field, theta, tof, hit);
+        if (bs) k_tof<float, RT_BSPLINE><<<nb, kBlock, 0, s>>>(G, (const CellBS<float>*)field, theta, tof, hit, sp.lanes);
+        else k_tof<float, RT_BILINEAR><<<nb, kBlock, 0, s>>>(G, (const CellCoef<float>*)field, theta, tof, hit, sp.lanes);
     }
     return cudaGetLastError();
 }
@@ -563,8 +628,8 @@ template <typename T> struct AdjOf<T, RT_BSPLINE> { using type = AdjSinkBSp<T>; 
 template <typename T, int I>
 __global__ void __launch_bounds__(kBlock, Occ<T, I>::blocks)
     k_adjoint(Geom G, const typename Samp<T, I>::Field* __restrict__ F, const double* theta, const double* g_tof,
-                 const double* tof_ref, double* g) {
-    const int slot = blockIdx.x * kBlock + threadIdx.x;
+                 const double* tof_ref, double* g, int lanes) {
+    const int slot = spread_slot(lanes);
     if (slot >= G.n_pairs) return;
     const int k = queue_pair(G, slot);
     const double w = g_tof[k] - (tof_ref ? tof_ref[k] : 0.0);
@@ -688,8 +753,9 @@ cudaError_t launch_adjoint_rows(const Geom& G, const void* field, const double* 
 template <typename T, int I>
 static void adjoint_impl(const Geom& G, const void* field, const double* theta, const double* g_tof,
                          const double* tof_ref, double* g_c, cudaStream_t s) {
-    k_adjoint<T, I><<<grid_for(G.n_pairs), kBlock, 0, s>>>(G, (const typename Samp<T, I>::Field*)field, theta,
-                                                             g_tof, tof_ref, g_c);
+    const Spread sp = spread_for(G.n_pairs, sizeof(T) == 8 ? RT_FP64 : RT_FP32_COMP);
+    k_adjoint<T, I><<<sp.blocks, kBlock, 0, s>>>(G, (const typename Samp<T, I>::Field*)field, theta, g_tof, tof_ref,
+                                                 g_c, sp.lanes);
 }
 
 cudaError_t launch_adjoint(const Geom& G, const void* field, int prec, const double* theta,
@@ -767,9 +833,10 @@ template <typename T> struct RowsOf<T, RT_BSPLINE> { using type = RowSinkBSp<T>;
 template <typename T, int I>
 __global__ void __launch_bounds__(kBlock) k_rows(Geom G, const typename Samp<T, I>::Field* __restrict__ F,
                                                  const double* theta, int64_t* row_ptr, int32_t* col,
-                                                 double* val, bool fill) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= G.n_pairs) return;
+                                                 double* val, bool fill, int lanes) {
+    const int slot = spread_slot(lanes);
+    if (slot >= G.n_pairs) return;
+    const int k = queue_pair(G, slot);
     LinkCtx L;
     typename RowsOf<T, I>::type sink;
     sink.nx = G.nx; sink.ny = G.ny; sink.col = col; sink.val = val; sink.fill = fill;
@@ -786,18 +853,19 @@ __global__ void __launch_bounds__(kBlock) k_rows(Geom G, const typename Samp<T, 
 cudaError_t launch_rows(const Geom& G, const void* field, int prec, const double* theta, int64_t* row_ptr,
                         int32_t* col, double* val, bool fill, cudaStream_t s) {
     if (G.n_pairs == 0) return cudaSuccess;
-    const int nb = grid_for(G.n_pairs);
+    const Spread sp = spread_for(G.n_pairs, prec);
+    const int nb = sp.blocks;
     const bool bs = G.interp == RT_BSPLINE;
     if (prec == RT_FP64) {
         if (bs) k_rows<double, RT_BSPLINE><<<nb, kBlock, 0, s>>>(G, (const CellBS<double>*)field, theta, row_ptr, col,
-                                                                 val, fill);
+                                                                 val, fill, sp.lanes);
         else k_rows<double, RT_BILINEAR><<<nb, kBlock, 0, s>>>(G, (const CellCoef<double>*)field, theta, row_ptr, col,
-                                                               val, fill);
+                                                               val, fill, sp.lanes);
     } else {
         if (bs) k_rows<float, RT_BSPLINE><<<nb, kBlock, 0, s>>>(G, (const CellBS<float>*)field, theta, row_ptr, col,
-                                                                val, fill);
+                                                                val, fill, sp.lanes);
         else k_rows<float, RT_BILINEAR><<<nb, kBlock, 0, s>>>(G, (const CellCoef<float>*)field, theta, row_ptr, col,
-                                                              val, fill);
+                                                              val, fill, sp.lanes);
     }
     return cudaGetLastError();
 }
