@@ -317,6 +317,21 @@ int rt_path_matrix(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt,
                    int64_t capacity, int64_t* nnz_out, void* stream);
 
 /*
+ * rt_path_record / rt_path_expand — rt_path_matrix in two calls that trace every
+ * ray once. rt_path_record writes row_ptr and nnz_out as rt_path_matrix does
+ * (it synchronises the stream to read nnz) and keeps every ray's cell visits in
+ * the caller's rec (cap runs per pair, len unused; a run's four numbers are the
+ * visit's weight sums, not rt_link_rows' node weights). rt_path_expand writes
+ * the nnz entries of col and val from it, the same values as rt_path_matrix.
+ * RT_ENOMEM (row_ptr and nnz valid) if a ray visits more than cap cells: use
+ * rt_path_matrix then. RT_FP32_COMP and RT_BILINEAR only (RT_EINVAL otherwise).
+ */
+int rt_path_record(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt, const double* theta,
+                   const rt_rows* rec, int64_t* row_ptr, int64_t* nnz_out, void* stream);
+int rt_path_expand(rt_ctx* ctx, const rt_problem* prob, const rt_rows* rec, const int64_t* row_ptr,
+                   int32_t* col, double* val, void* stream);
+
+/*
  * rt_status_counts — synchronises `stream` and copies the per-status pair
  * counts of the last rt_link on this context: counts[s] for s = 0..7 (HOST
  * array), plus counts[7] = total RK4 steps taken by that call. Returns RT_OK

@@ -267,6 +267,9 @@ def rt_tof_adjoint(prob: Problem, theta: torch.Tensor, g_tof: torch.Tensor, ds: 
     return g
 
 
+RECORD_BYTES = 16 << 30   # most memory rt_path_matrix takes for the recorded visits
+
+
 def rt_path_matrix(prob: Problem, theta: torch.Tensor, ds: float, precision: str = "fp32c",
                    ctx: Optional[Context] = None, stream=None, integrator: str = "rk4",
                    c: Optional[torch.Tensor] = None, interpolator: str = "bilinear"):
@@ -280,6 +283,30 @@ def rt_path_matrix(prob: Problem, theta: torch.Tensor, ds: float, precision: str
     ps = prob.struct(c)
     o = _opts(ds, precision=precision, integrator=integrator, interpolator=interpolator)
     th = theta.contiguous()
+    # one trace per ray: its cell visits are kept while the matrix is laid out
+    # (a third of the time of counting, counting and filling by three traces).
+    # The visits take about as much memory as the matrix, hence the limit.
+    cap = ctx.lib.rt_rows_cap(C.byref(ps))
+    size = prob.n_pairs * cap * _L.RUN_BYTES
+    if precision == "fp32c" and interpolator == "bilinear" and 0 < size <= RECORD_BYTES:
+        try:
+            runs = torch.empty(size, dtype=torch.uint8, device=dev)
+        except torch.OutOfMemoryError:
+            runs = None
+        if runs is not None:
+            rec = _L.RtRows(runs.data_ptr(), None, cap)
+            rc = ctx.lib.rt_path_record(ctx.h, C.byref(ps), C.byref(o), _ptr(th), C.byref(rec), _ptr(row_ptr),
+                                        C.byref(nnz), _stream(stream))
+            if rc == _L.RT_OK:
+                col = torch.empty(max(nnz.value, 1), dtype=torch.int32, device=dev)
+                val = torch.empty(max(nnz.value, 1), dtype=torch.float64, device=dev)
+                _L.check(ctx.h, ctx.lib.rt_path_expand(ctx.h, C.byref(ps), C.byref(rec), _ptr(row_ptr), _ptr(col),
+                                                       _ptr(val), _stream(stream)))
+                if stream is not None:
+                    runs.record_stream(stream)   # freed below, still read there
+                return row_ptr, col[: nnz.value], val[: nnz.value]
+            if rc != _L.RT_ENOMEM:
+                _L.check(ctx.h, rc)
     rc = ctx.lib.rt_path_matrix(ctx.h, C.byref(ps), C.byref(o), _ptr(th), _ptr(row_ptr), None, None, 0,
                                 C.byref(nnz), _stream(stream))
     if rc not in (_L.RT_OK, _L.RT_ENOMEM):

@@ -23,7 +23,7 @@ EXPORTED = [
     "rt_tof_forward_noalloc", "rt_batch_run", "rtborn_maps", "rtborn_apply", "rtborn_adjoint",
     "rt_csr_matvec", "rt_csr_rmatvec", "rt_bspline_coef", "rtborn_maps_abs", "rtborn_apply_abs",
     "rtborn_adjoint_abs", "rt_peak_fma", "rt_peak_gather", "rt_peak_read", "rt_wait_selftest", "rt_rows_cap",
-    "rt_link_rows", "rt_tof_adjoint_rows",
+    "rt_link_rows", "rt_tof_adjoint_rows", "rt_path_record", "rt_path_expand",
 ]
 RTBORN_GEMM_FP32, RTBORN_GEMM_TF32X3 = 0, 1
 ABI_VERSION = 4   # layout of RtOptions below
@@ -103,6 +103,8 @@ def load():
         L.rt_tof_adjoint.argtypes = [vp, P(RtProblem), P(RtOptions), vp, vp, vp, vp, vp]
         L.rt_path_matrix.argtypes = [vp, P(RtProblem), P(RtOptions), vp, vp, vp, vp, C.c_int64,
                                      P(C.c_int64), vp]
+        L.rt_path_record.argtypes = [vp, P(RtProblem), P(RtOptions), vp, P(RtRows), vp, P(C.c_int64), vp]
+        L.rt_path_expand.argtypes = [vp, P(RtProblem), P(RtRows), vp, vp, vp, vp]
         L.rt_status_counts.argtypes = [vp, P(C.c_int64), vp]
         L.rt_tof_forward_noalloc.argtypes = [P(RtProblem), P(RtOptions), vp, vp, vp, vp]
         L.rt_batch_run.argtypes = [vp, C.c_int32, P(RtInstance), P(RtOptions), vp]

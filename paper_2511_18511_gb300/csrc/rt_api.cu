@@ -392,6 +392,26 @@ int rt_tof_adjoint(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt, c
     return e == cudaSuccess ? RT_OK : cuda_fail(ctx, e, "adjoint kernel");
 }
 
+// Row lengths row_ptr[1..n] to row ends, in place.
+static int scan_rows(rt_ctx* ctx, int n, int64_t* row_ptr, cudaStream_t s) {
+    if (n <= 0) return RT_OK;
+    size_t need = 0;
+    cudaError_t e = rt::launch_scan(row_ptr, n, nullptr, &need, s);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "scan size");
+    if (ctx->scan_bytes < need) {
+        if (ctx->scan_tmp) cudaFree(ctx->scan_tmp);
+        ctx->scan_tmp = nullptr;
+        ctx->scan_bytes = 0;
+        e = cudaMalloc(&ctx->scan_tmp, need);
+        if (e != cudaSuccess) return fail(ctx, RT_ENOMEM, "scan workspace");
+        ctx->scan_bytes = need;
+    }
+    size_t have = ctx->scan_bytes;
+    e = rt::launch_scan(row_ptr, n, ctx->scan_tmp, &have, s);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "scan");
+    return RT_OK;
+}
+
 int rt_path_matrix(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt, const double* theta,
                    int64_t* row_ptr, int32_t* col, double* val, int64_t capacity, int64_t* nnz_out,
                    void* stream) {
@@ -405,22 +425,8 @@ int rt_path_matrix(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt, c
     if (e != cudaSuccess) return cuda_fail(ctx, e, "row_ptr reset");
     e = rt::launch_rows(G, ctx->field, opt->precision, theta, row_ptr, nullptr, nullptr, false, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "row count kernel");
-    if (G.n_pairs > 0) {
-        size_t need = 0;
-        e = rt::launch_scan(row_ptr, G.n_pairs, nullptr, &need, s);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "scan size");
-        if (ctx->scan_bytes < need) {
-            if (ctx->scan_tmp) cudaFree(ctx->scan_tmp);
-            ctx->scan_tmp = nullptr;
-            ctx->scan_bytes = 0;
-            e = cudaMalloc(&ctx->scan_tmp, need);
-            if (e != cudaSuccess) return fail(ctx, RT_ENOMEM, "scan workspace");
-            ctx->scan_bytes = need;
-        }
-        size_t have = ctx->scan_bytes;
-        e = rt::launch_scan(row_ptr, G.n_pairs, ctx->scan_tmp, &have, s);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "scan");
-    }
+    rc = scan_rows(ctx, G.n_pairs, row_ptr, s);
+    if (rc) return rc;
     int64_t nnz = 0;
     e = cudaMemcpyAsync(&nnz, row_ptr + G.n_pairs, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -429,6 +435,56 @@ int rt_path_matrix(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt, c
     if (capacity < nnz || !col || !val) return fail(ctx, RT_ENOMEM, "capacity smaller than nnz (row_ptr is valid)");
     e = rt::launch_rows(G, ctx->field, opt->precision, theta, row_ptr, col, val, true, s);
     return e == cudaSuccess ? RT_OK : cuda_fail(ctx, e, "row fill kernel");
+}
+
+int rt_path_record(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt, const double* theta, const rt_rows* rec,
+                   int64_t* row_ptr, int64_t* nnz_out, void* stream) {
+    cudaStream_t s = (cudaStream_t)stream;
+    if (!ctx) return RT_EINVAL;
+    if (!row_ptr || !nnz_out) return fail(ctx, RT_EINVAL, "row_ptr and nnz_out are required");
+    if (!theta && prob && prob->n_pairs > 0) return fail(ctx, RT_EINVAL, "theta is required");
+    if (!opt) return fail(ctx, RT_EINVAL, "options pointer is NULL");
+    if (opt->precision != RT_FP32_COMP || opt->interpolator != RT_BILINEAR)
+        return fail(ctx, RT_EINVAL, "recorded rows need RT_FP32_COMP and RT_BILINEAR");
+    if (!rec || rec->cap < 1 || (prob && prob->n_pairs > 0 && !rec->runs))
+        return fail(ctx, RT_EINVAL, "rows: runs and cap >= 1 are required");
+    rt::Geom G;
+    int rc = prepare(ctx, prob, opt, false, s, &G);
+    if (rc) return rc;
+    cudaError_t e = cudaMemsetAsync(row_ptr, 0, sizeof(int64_t), s);
+    if (e == cudaSuccess)
+        e = rt::launch_rows_record(G, ctx->field, theta, row_ptr, rt::RowRec{rec->runs, nullptr, rec->cap}, s);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "row record kernel");
+    rc = scan_rows(ctx, G.n_pairs, row_ptr, s);
+    if (rc) return rc;
+    int64_t over = 0, nnz = 0;
+    e = cudaMemcpyAsync(&over, row_ptr, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&nnz, row_ptr + G.n_pairs, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "nnz readback");
+    if (over) {
+        e = cudaMemsetAsync(row_ptr, 0, sizeof(int64_t), s);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "row_ptr reset");
+        if (G.n_pairs == 0) nnz = 0;
+    }
+    *nnz_out = nnz;
+    return over ? fail(ctx, RT_ENOMEM, "a row visits more than cap cells (row_ptr is valid)") : RT_OK;
+}
+
+int rt_path_expand(rt_ctx* ctx, const rt_problem* prob, const rt_rows* rec, const int64_t* row_ptr, int32_t* col,
+                   double* val, void* stream) {
+    if (!ctx) return RT_EINVAL;
+    ctx->err.clear();
+    if (!prob || prob->n_pairs < 0 || prob->grid.nx < 3) return fail(ctx, RT_EINVAL, "problem invalid");
+    if (prob->n_pairs == 0) return RT_OK;
+    if (!rec || rec->cap < 1 || !rec->runs || !row_ptr || !col || !val)
+        return fail(ctx, RT_EINVAL, "rows, row_ptr, col and val are required");
+    int rc = set_device(ctx);
+    if (rc) return rc;
+    const cudaError_t e = rt::launch_rows_expand(prob->n_pairs, prob->grid.nx, row_ptr,
+                                                 rt::RowRec{rec->runs, nullptr, rec->cap}, col, val, (cudaStream_t)stream);
+    return e == cudaSuccess ? RT_OK : cuda_fail(ctx, e, "row expand kernel");
 }
 
 int rt_status_counts(rt_ctx* ctx, int64_t counts[8], void* stream) {

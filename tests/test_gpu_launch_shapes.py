@@ -1,7 +1,10 @@
-"""The launches that spread few rays over many warps and the step forms that the
-FP32 march chooses by the lanes at work: every form gives the same bits, since
-a ray's arithmetic does not depend on the lane or the warp's other rays.
+"""The launches that spread few rays over many warps, the step forms that the
+FP32 march chooses by the lanes at work, and the system matrix from one trace:
+every form gives the same bits, since a ray's arithmetic does not depend on
+the lane, the warp's other rays or the kernel that runs it.
 """
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -58,3 +61,35 @@ def test_forward_is_the_same_on_any_number_of_lanes(rt, precision, interpolator,
         sub = rt.Problem(prob.grid, prob.c, prob.tx, prob.ring_radius, pairs[sel].contiguous())
         t, hit = rt.rt_tof_forward(sub, theta[sel].contiguous(), ds, **how)
         assert torch.equal(t, t_all[sel]) and torch.equal(hit, hit_all[sel])
+
+
+@pytest.mark.parametrize("integrator", ["rk4", "heun"])
+@pytest.mark.parametrize("n_tx", [2, 40, 128])
+def test_path_matrix_from_one_trace(rt, n_tx, integrator, monkeypatch):
+    prob = _problem(rt, n_tx)
+    _, theta = _straight(prob)
+    ds = 0.1 * prob.grid.h
+    one = rt.rt_path_matrix(prob, theta, ds, integrator=integrator)
+    monkeypatch.setattr(rt, "RECORD_BYTES", 0)     # count, count and fill
+    three = rt.rt_path_matrix(prob, theta, ds, integrator=integrator)
+    for a, b in zip(one, three):
+        assert torch.equal(a, b)
+
+
+def test_path_record_reports_rows_longer_than_its_capacity(rt):
+    from paper_2511_18511_gb300 import _lib as L
+    prob = _problem(rt, 24)
+    _, theta = _straight(prob)
+    ds = 0.1 * prob.grid.h
+    want = rt.rt_path_matrix(prob, theta, ds)
+    ctx = rt.default_context(prob.c.device.index)
+    cap = 8                                        # most rows visit more cells
+    runs = torch.empty(prob.n_pairs * cap * L.RUN_BYTES, dtype=torch.uint8, device="cuda")
+    row_ptr = torch.full((prob.n_pairs + 1,), -1, dtype=torch.int64, device="cuda")
+    nnz = C.c_int64(-1)
+    ps, o, rec = prob.struct(), rt._opts(ds), L.RtRows(runs.data_ptr(), None, cap)
+    s = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    rc = ctx.lib.rt_path_record(ctx.h, C.byref(ps), C.byref(o), C.c_void_p(theta.data_ptr()), C.byref(rec),
+                                C.c_void_p(row_ptr.data_ptr()), C.byref(nnz), s)
+    assert rc == L.RT_ENOMEM and nnz.value == want[1].numel()
+    assert torch.equal(row_ptr, want[0])
