@@ -388,8 +388,8 @@ typedef struct {
  * L2 misfit (rt_tof_adjoint with g_tof = T), for n_inst problems of different
  * grids and rings in ONE persistent launch over all their pairs (longest rings
  * first, longest chords first within a ring). Each pair is linked (paper
- * Sec. 3.4) and then retraced by the same lane with its adjoint weight
- * T - T_ref (Sec. 3.1.1), so forward and adjoint share one launch.
+ * Sec. 3.4) and then, in a second launch, retraced with its adjoint weight
+ * T - T_ref (Sec. 3.1.1).
  *   inst   HOST array of n_inst descriptors (read during the call).
  * Every per-instance output is as for rt_link / rt_tof_adjoint; status counts
  * (summed over instances) are read with rt_status_counts. The call sizes the

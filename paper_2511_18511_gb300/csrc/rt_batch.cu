@@ -1,8 +1,7 @@
-// rt_batch.cu — many ToF problems (uneven grids and rings) in one persistent
-// launch: every pair of every instance is linked and, when the instance has
-// measured travel times, retraced right away by the same lane with the
-// adjoint weight w = T - T_ref (the gradient of 0.5*||T - T_ref||^2), so the
-// forward and the adjoint share one launch and one tail.
+// rt_batch.cu — many ToF problems (uneven grids and rings) in three launches
+// over all instances: their fans, the persistent link of every pair and, for
+// instances with measured travel times, the retrace of every pair with the
+// adjoint weight w = T - T_ref (the gradient of 0.5*||T - T_ref||^2).
 #include <algorithm>
 #include <climits>
 #include <atomic>
@@ -31,51 +30,8 @@ struct InstDesc {
     long long pair_base;    // first global queue slot of this instance
 };
 
-// Adjoint sink that a lane switches on only for its adjoint retrace, so
-// linking and adjoint lanes share one instruction stream. Only the running
-// cell accumulation lives in registers; the target, weight and grid size sit
-// in the lane's shared linking state and are read when a cell is flushed.
-template <typename T>
-struct GatedAdjSink {
-    bool on;
-    LinkState* L;
-    CellAcc<T> acc;
-    __device__ __forceinline__ void flush() {
-        if (acc.ai == INT_MIN) return;
-        const T w = (T)L->adj_w;
-        const int nx = L->adj_nx, ny = L->adj_ny;
-        const T w11 = acc.Wxy, w10 = acc.Wx - acc.Wxy, w01 = acc.Wy - acc.Wxy;
-        const T w00 = (acc.W - acc.Wx) - w01;
-        const int i = min(max(acc.ai, 0), nx - 2), j = min(max(acc.aj, 0), ny - 2);
-        double* p = L->adj_g + (size_t)j * nx + i;
-        atomicAdd(p, to_double(w * w00));
-        atomicAdd(p + 1, to_double(w * w10));
-        atomicAdd(p + nx, to_double(w * w01));
-        atomicAdd(p + nx + 1, to_double(w * w11));
-    }
-    __device__ __forceinline__ void add(int ci, int cj, T tx, T ty, T a) {
-        if (!on) return;
-        if (ci != acc.ai || cj != acc.aj) {
-            flush();
-            acc.reset();
-            acc.ai = ci;
-            acc.aj = cj;
-        }
-        acc.W += a;
-        acc.Wx += a * tx;
-        acc.Wy += a * ty;
-        acc.Wxy += a * tx * ty;
-    }
-    __device__ __forceinline__ void finish() {
-        if (!on) return;
-        flush();
-        acc.reset();
-    }
-};
-
 // All instance descriptors travel as one kernel parameter (read through the
 // constant cache, so the geometry costs no registers); 64 instances per launch.
-constexpr int kMaxBatch = 64;
 struct BatchParams {
     int n_inst;
     InstDesc d[kMaxBatch];
@@ -105,10 +61,7 @@ __global__ void __launch_bounds__(BLOCK, MINB)
     Cell<T> C;
     C.F = nullptr; C.nx = 3; C.ny = 3; C.pi = INT_MIN; C.pj = INT_MIN;
     TraceState<T> ts;
-    GatedAdjSink<T> sink;
-    sink.on = false;
-    sink.L = &L;
-    sink.acc.reset();
+    NoSink sink;
     long long steps = 0;
     unsigned n_ok = 0, n_max = 0, n_cap = 0, n_bad = 0;
     bool active = false;
@@ -167,7 +120,6 @@ __global__ void __launch_bounds__(BLOCK, MINB)
                 pair_of(G, k, e, r);
                 fan_start(G, L, d.fan + (size_t)e * fan_rays, fan_rays);
             }
-            sink.on = false;
             trace_begin(ts, G, L.xe, L.ye, L.next);
             active = true;
         }
@@ -184,11 +136,6 @@ __global__ void __launch_bounds__(BLOCK, MINB)
         if (!ended) continue;
         const TraceOut o = trace_end(C, G, ts, L.xe, L.ye, L.xr, L.yr, sink);
         steps += o.steps;
-        if (sink.on) {                    // adjoint retrace done
-            sink.on = false;
-            active = false;
-            continue;
-        }
         if (link_update(G, L, o, tol, max_iter, fan_rays >= 2 ? d.fan : nullptr, fan_rays)) {
             const int k = L.k;
             const int st = (L.best_d2 <= tol * tol) ? RT_RAY_OK
@@ -201,18 +148,7 @@ __global__ void __launch_bounds__(BLOCK, MINB)
             n_ok += st == RT_RAY_OK;
             n_max += st == RT_RAY_MAXITER;
             n_cap += st == RT_RAY_STEPCAP;
-            const double w = d.tof_ref ? L.best_T - d.tof_ref[k] : 0.0;
-            if (d.tof_ref && w != 0.0 && isfinite(w)) {
-                sink.on = true;
-                L.adj_g = d.g;
-                L.adj_w = w;
-                L.adj_nx = G.nx;
-                L.adj_ny = G.ny;
-                sink.acc.reset();
-                trace_begin(ts, G, L.xe, L.ye, L.best_th);
-            } else {
-                active = false;
-            }
+            active = false;
         } else {
             trace_begin(ts, G, L.xe, L.ye, L.next);
         }
@@ -231,6 +167,45 @@ __global__ void __launch_bounds__(BLOCK, MINB)
             atomicAdd(&counters[7], v[4]);
         }
     }
+}
+
+// Adjoint scatter of every linked pair of every instance, one thread per pair
+// in the link's queue order: a warp retraces parallel rays of equal length. As
+// a retrace inside k_batch, on whichever lane had linked the pair, it shared
+// the loop with unrelated linking rays and its sink cost the link registers:
+// eight instances of up to 768^2 nodes and 256 transducers took 31.2 ms then,
+// 24.5 ms now (25.3 ms at 5 blocks an SM in place of 4, 26.6 ms at 6).
+template <typename T>
+__global__ void __launch_bounds__(128, LinkOcc<T>::blocks)
+    k_batch_adjoint(const __grid_constant__ BatchParams P, long long total, unsigned long long* counters, int lanes) {
+    const int lane = threadIdx.x & 31;
+    const long long q = ((blockIdx.x * 128ll + threadIdx.x) >> 5) * lanes + lane;
+    unsigned long long steps = 0;
+    if (lane < lanes && q < total) {
+        const InstDesc& d = P.d[find_inst(P, q)];
+        const Geom& G = d.G;
+        const int k = queue_pair(G, (int)(q - d.pair_base));
+        const double w = d.tof_ref ? d.tof[k] - d.tof_ref[k] : 0.0;
+        LinkCtx X;
+        if (w != 0.0 && isfinite(w) && setup_pair(G, k, X)) {
+            Cell<T> C;
+            C.F = static_cast<const CellCoef<T>*>(d.field);
+            C.nx = G.nx;
+            C.ny = G.ny;
+            C.pi = INT_MIN;
+            C.pj = INT_MIN;
+            AdjSink<T> sink;
+            sink.g = d.g;
+            sink.nx = G.nx;
+            sink.ny = G.ny;
+            sink.init();
+            sink.w = (T)w;
+            steps = (unsigned long long)trace_ray<T>(C, G, X.xe, X.ye, d.theta[k], X.xr, X.yr, sink).steps;
+        }
+    }
+    __syncwarp();
+    for (int off = 16; off > 0; off >>= 1) steps += __shfl_down_sync(0xffffffffu, steps, off);
+    if (lane == 0 && steps) atomicAdd(&counters[7], steps);
 }
 
 // g_c = -1000 g / c^2 for every instance with an adjoint (blockIdx.y = instance).
@@ -369,6 +344,8 @@ extern "C" int rt_batch_run(rt_ctx* ctx, int32_t n_inst, const rt_instance* inst
     if (cudaSetDevice(ctx->device) != cudaSuccess) return rt::set_error(ctx, RT_ECUDA, "cudaSetDevice");
     unsigned char* ws = static_cast<unsigned char*>(ctx->batch_ws);
     cudaError_t e = cudaMemsetAsync(ctx->counters, 0, 8 * sizeof(unsigned long long), s);
+    rt::FanBatch fans{};
+    long long fan_total = 0;
     for (int slot = 0; slot < n_inst && e == cudaSuccess; ++slot) {
         const rt_instance& I = inst[order[(size_t)slot]];
         InstDesc& d = D[(size_t)slot];
@@ -379,9 +356,9 @@ extern "C" int rt_batch_run(rt_ctx* ctx, int32_t n_inst, const rt_instance* inst
         if (e != cudaSuccess) break;
         if (opt->fan_rays >= 2 && I.prob.n_pairs > 0) {
             d.fan = reinterpret_cast<const double*>(ws + fan_off[slot]);
-            e = rt::launch_fan(d.G, opt->fan_ds_mm, d.field, opt->precision, opt->fan_rays, I.theta_io,
-                               reinterpret_cast<double*>(ws + fan_off[slot]), reinterpret_cast<int*>(ws + need_off[slot]),
-                               ctx->counters, s);
+            e = rt::fan_job(d.G, opt->fan_ds_mm, d.field, opt->fan_rays, I.theta_io,
+                            reinterpret_cast<double*>(ws + fan_off[slot]), reinterpret_cast<int*>(ws + need_off[slot]),
+                            fans, fan_total, s);
             if (e != cudaSuccess) break;
         }
         d.theta = I.theta_io;
@@ -395,6 +372,7 @@ extern "C" int rt_batch_run(rt_ctx* ctx, int32_t n_inst, const rt_instance* inst
         if (I.tof_ref)
             e = cudaMemsetAsync(I.g_c, 0, sizeof(double) * (size_t)I.prob.grid.nx * I.prob.grid.ny, s);
     }
+    if (e == cudaSuccess) e = rt::launch_fan_batch(fans, fan_total, opt->precision, opt->fan_rays, ctx->counters, s);
     if (e != cudaSuccess) return rt::set_error(ctx, RT_ECUDA, std::string("batch set-up: ") + cudaGetErrorString(e));
     rt::BatchParams params{};   // the kernel parameter, copied at launch
     params.n_inst = n_inst;
@@ -407,6 +385,15 @@ extern "C" int rt_batch_run(rt_ctx* ctx, int32_t n_inst, const rt_instance* inst
     if (!ok)
         return rt::set_error(ctx, RT_EINVAL, "unsupported block_threads / step_unroll / blocks_per_sm combination");
     if (e != cudaSuccess) return rt::set_error(ctx, RT_ECUDA, std::string("batch kernel: ") + cudaGetErrorString(e));
+    bool adjoint = false;
+    for (const InstDesc& d : D) adjoint |= d.tof_ref != nullptr;
+    if (adjoint && total > 0) {
+        const rt::Spread sp = rt::spread_for(total, opt->precision);
+        if (opt->precision == RT_FP64)
+            rt::k_batch_adjoint<double><<<sp.blocks, 128, 0, s>>>(params, total, ctx->counters, sp.lanes);
+        else
+            rt::k_batch_adjoint<float><<<sp.blocks, 128, 0, s>>>(params, total, ctx->counters, sp.lanes);
+    }
     rt::k_batch_finish<<<dim3(64, (unsigned)n_inst), 256, 0, s>>>(params);
     e = cudaGetLastError();
     if (e != cudaSuccess) return rt::set_error(ctx, RT_ECUDA, std::string("batch finish: ") + cudaGetErrorString(e));

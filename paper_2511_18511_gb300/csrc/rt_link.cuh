@@ -72,10 +72,6 @@ struct LinkState {
     int fan_k0;                      // fan start: interval between rays fan_k0, fan_k0 + 1 whose
                                      // four surrounding rays are usable for the second angle; else -1;
                                      // -2: the pair did not start from the fan
-    // adjoint retrace of the batched kernel (read on flushes only)
-    double* adj_g;
-    double adj_w;
-    int adj_nx, adj_ny;
 };
 
 __device__ __forceinline__ void br_insert(LinkState& L, double t, double m) {
@@ -571,6 +567,26 @@ struct Spread {
     int lanes, blocks;
 };
 Spread spread_for(long long n, int prec);
+
+// The fans of a batch's instances, one launch (k_fan_batch): a kernel parameter.
+constexpr int kMaxBatch = 64;
+struct FanJob {
+    Geom G;            // with the fan's step
+    const void* field;
+    const int* need;
+    double* fan;
+    double margin;
+    long long base;    // first ray of this instance
+};
+struct FanBatch {
+    int n;
+    FanJob job[kMaxBatch];
+};
+// Adds an instance's fan to B (marking the emitters that need it) and its rays to `rays`.
+cudaError_t fan_job(const Geom& G, double fan_ds, const void* field, int fan_rays, const double* theta, double* fan,
+                    int* fan_need, FanBatch& B, long long& rays, cudaStream_t s);
+cudaError_t launch_fan_batch(const FanBatch& B, long long rays, int prec, int fan_rays, unsigned long long* counters,
+                             cudaStream_t s);
 
 // Recording target of a linking launch (rt_link_rows); runs == null: none.
 struct RowRec {

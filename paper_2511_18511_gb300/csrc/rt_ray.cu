@@ -242,6 +242,28 @@ __global__ void __launch_bounds__(kBlock) k_fan(Geom G, const typename Samp<T, I
     count_steps(steps, counters);
 }
 
+// The fans of all instances of a batch in one launch: alone, the fan of one
+// instance leaves most of the GPU idle for as long as its longest ray takes
+// (eight instances: 35.8 -> 31.2 ms for the whole call).
+template <typename T>
+__global__ void __launch_bounds__(kBlock) k_fan_batch(const __grid_constant__ FanBatch B, long long rays, int K,
+                                                      unsigned long long* counters, int lanes) {
+    const int lane = threadIdx.x & 31;
+    const long long slot = ((blockIdx.x * (long long)kBlock + threadIdx.x) >> 5) * lanes + lane;
+    long long steps = 0;
+    if (lane < lanes && slot < rays) {
+        int lo = 0, hi = B.n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (B.job[mid].base <= slot) lo = mid; else hi = mid - 1;
+        }
+        const FanJob& J = B.job[lo];
+        steps = fan_ray<T, RT_BILINEAR>(J.G, (const CellCoef<T>*)J.field, K, J.margin, J.need, J.fan,
+                                        (int)(slot - J.base));
+    }
+    count_steps(steps, counters);
+}
+
 // Persistent linking kernel: each lane takes pairs from the queue, advances
 // its own trace up to kLinkSteps RK4 steps per loop iteration, and updates the
 // linking state when a trace ends, so lanes never wait for other lanes' pairs
@@ -439,6 +461,28 @@ static cudaError_t mark_fans(const Geom& G, const double* theta, int* fan_need, 
     cudaError_t e = cudaMemsetAsync(fan_need, 0, sizeof(int) * (size_t)G.n_tx, s);
     if (e != cudaSuccess) return e;
     k_fan_mark<<<grid_for(G.n_pairs), kBlock, 0, s>>>(G, theta, fan_need);
+    return cudaGetLastError();
+}
+
+cudaError_t fan_job(const Geom& G, double fan_ds, const void* field, int fan_rays, const double* theta, double* fan,
+                    int* fan_need, FanBatch& B, long long& rays, cudaStream_t s) {
+    FanJob& J = B.job[B.n++];
+    J.G = fan_ds > 0.0 ? with_step(G, fan_ds) : G;
+    J.field = field;
+    J.need = fan_need;
+    J.fan = fan;
+    J.margin = fan_margin(G);
+    J.base = rays;
+    rays += (long long)G.n_tx * fan_rays;
+    return mark_fans(G, theta, fan_need, s);
+}
+
+cudaError_t launch_fan_batch(const FanBatch& B, long long rays, int prec, int fan_rays, unsigned long long* counters,
+                             cudaStream_t s) {
+    if (rays == 0) return cudaSuccess;
+    const Spread sp = spread_for(rays, prec);
+    if (prec == RT_FP64) k_fan_batch<double><<<sp.blocks, kBlock, 0, s>>>(B, rays, fan_rays, counters, sp.lanes);
+    else k_fan_batch<float><<<sp.blocks, kBlock, 0, s>>>(B, rays, fan_rays, counters, sp.lanes);
     return cudaGetLastError();
 }
 

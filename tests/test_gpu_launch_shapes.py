@@ -93,3 +93,25 @@ def test_path_record_reports_rows_longer_than_its_capacity(rt):
                                 C.c_void_p(row_ptr.data_ptr()), C.byref(nnz), s)
     assert rc == L.RT_ENOMEM and nnz.value == want[1].numel()
     assert torch.equal(row_ptr, want[0])
+
+
+def test_batch_of_several_is_each_alone(rt):
+    """The instances' fans and adjoints run in one launch each; a batch of one
+    gives the same bits, up to the order of the adjoint's FP64 sums (at most
+    the 64 x 4 additions to a node here, 2^-53 of the sum of magnitudes each)."""
+    probs = [_problem(rt, n, nx, ny, h) for n, nx, ny, h in ((33, 101, 96, 0.5), (2, 64, 70, 0.4), (70, 130, 128, 0.25))]
+
+    def instances():
+        out = []
+        for p in probs:
+            pairs, _ = _straight(p)
+            d = (p.tx[pairs[:, 0].long()] - p.tx[pairs[:, 1].long()]).norm(dim=1)
+            out.append(rt.BatchInstance.create(p, (d / 1.6).contiguous()))   # all weights of one sign: no cancellation
+        return out
+
+    batch = rt.rt_batch_run(instances(), 0.03, fan_ds=0.1)
+    for b, alone in zip(batch, instances()):
+        rt.rt_batch_run([alone], 0.03, fan_ds=0.1)
+        for name in ("theta", "tof", "hit", "status", "iters"):
+            assert torch.equal(getattr(b, name), getattr(alone, name))
+        assert ((b.g_c - alone.g_c).abs() <= 1e-11 * alone.g_c.abs()).all()
