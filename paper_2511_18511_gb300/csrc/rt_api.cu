@@ -227,6 +227,8 @@ int make_geom(rt_ctx* ctx, const rt_problem* p, const rt_options* o, Geom* G) {
     G->Hf = (float)(o->ds_mm / g.h_mm);
     G->dsf = (float)o->ds_mm;
     G->Rcf = (float)Rc;
+    G->Hd = o->ds_mm / g.h_mm;
+    G->Rcd = Rc;
     G->oxff = (float)G->oxf;
     G->oyff = (float)G->oyf;
     G->qf = (float)G->q;

@@ -449,6 +449,7 @@ Geom with_step(const Geom& G, double ds) {
     F.ds = ds;
     F.dsf = (float)ds;
     F.Hf = (float)(ds / G.h);
+    F.Hd = ds / G.h;
     F.max_steps = (long long)std::ceil(8.0 * G.R / ds);
     F.max_steps_i = (int)F.max_steps;
     return F;

@@ -69,6 +69,7 @@ struct Geom {
     const double* tx_phi;   // [n_tx] polar angle of each transducer, NaN if off the ring; null = compute
     // FP32 copies of the per-step constants, so the FP32 march issues no FP64
     float Hf, dsf, Rcf, oxff, oyff, qf;
+    double Hd, Rcd;         // ds / h and R / h
     int Qi;                 // Q as 32-bit (grids up to 32k cells per side)
 };
 
@@ -83,9 +84,9 @@ template <> struct StepK<float> {
     __device__ __forceinline__ static float q(const Geom& G) { return G.qf; }
 };
 template <> struct StepK<double> {
-    __device__ __forceinline__ static double H(const Geom& G) { return G.ds / G.h; }
+    __device__ __forceinline__ static double H(const Geom& G) { return G.Hd; }
     __device__ __forceinline__ static double ds(const Geom& G) { return G.ds; }
-    __device__ __forceinline__ static double Rc(const Geom& G) { return G.R / G.h; }
+    __device__ __forceinline__ static double Rc(const Geom& G) { return G.Rcd; }
     __device__ __forceinline__ static double oxf(const Geom& G) { return G.oxf; }
     __device__ __forceinline__ static double oyf(const Geom& G) { return G.oyf; }
     __device__ __forceinline__ static double q(const Geom& G) { return G.q; }
@@ -109,7 +110,25 @@ __device__ __forceinline__ float rcp_approx(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-__device__ __forceinline__ double rcp_approx(double x) { return 1.0 / x; }
+// In FP64 the hardware's approximation refined by two Newton steps, each of
+// which squares the error: 4 FP64 operations against a division's 8 or more, on
+// a part whose FP64 rate is 1/64 of FP32. The sound speed is a normal number.
+__device__ __forceinline__ double rcp_approx(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+
+// 0 <= u, v < 1 on the bits: those of a non-negative number below 1 are below
+// 1's, those of a negative one (-0 too) or NaN are not. In FP64 the high words
+// decide, which keeps the test off the FP64 pipe.
+__device__ __forceinline__ bool in_unit(float u, float v) {
+    return max(__float_as_uint(u), __float_as_uint(v)) < 0x3f800000u;
+}
+__device__ __forceinline__ bool in_unit(double u, double v) {
+    return max((unsigned)__double2hiint(u), (unsigned)__double2hiint(v)) < 0x3ff00000u;
+}
 
 // Two FP32 values in one 64-bit register pair. Each operation below is one
 // instruction that rounds both halves exactly as its scalar form does, so the
@@ -157,7 +176,7 @@ __device__ __forceinline__ F2 sub2(F2 a, F2 b) {
 template <typename T>
 __device__ __forceinline__ bool cell_locate(int ci, int cj, T u, T v, int pi, int pj, int& i, int& j, T& tx,
                                             T& ty) {
-    if (ci == pi && cj == pj && u >= (T)0 && u < (T)1 && v >= (T)0 && v < (T)1) {
+    if (ci == pi && cj == pj && in_unit(u, v)) {
         tx = u;
         ty = v;
         return false;
@@ -344,9 +363,18 @@ template <> struct Dir<double> {
     __device__ __forceinline__ void add_normalize(double ix, double iy) {
         x += ix;
         y += iy;
-        double n = sqrt(x * x + y * y);
-        x /= n;
-        y /= n;
+        // |d|^2 = 1 + e: 1/sqrt(1 + e) by its series, whose next term is below
+        // 3e-17 here, in place of a root and two divisions
+        const double e = fma(x, x, fma(y, y, -1.0));
+        if (fabsf((float)e) < 1e-4f) {
+            const double k = e * fma(e, fma(e, -0.3125, 0.375), -0.5);
+            x = fma(x, k, x);
+            y = fma(y, k, y);
+        } else {
+            const double n = sqrt(x * x + y * y);
+            x /= n;
+            y /= n;
+        }
     }
     __device__ __forceinline__ double dx() const { return x; }
     __device__ __forceinline__ double dy() const { return y; }
@@ -447,16 +475,23 @@ __device__ __forceinline__ void rk4_step(CellT& C, const RayState<T>& S, T H, Ra
     T nfx = S.fx, nfy = S.fy;
     N.lx = S.lx;
     N.ly = S.ly;
-    add_frac(nfx, N.lx, H6 * (dx + (T)2 * (e2x + e3x) + e4x) + H * S.d.lx());
-    add_frac(nfy, N.ly, H6 * (dy + (T)2 * (e2y + e3y) + e4y) + H * S.d.ly());
+    if constexpr (sizeof(T) == 8) {
+        nfx += H6 * (dx + (T)2 * (e2x + e3x) + e4x);
+        nfy += H6 * (dy + (T)2 * (e2y + e3y) + e4y);
+    } else {
+        add_frac(nfx, N.lx, H6 * (dx + (T)2 * (e2x + e3x) + e4x) + H * S.d.lx());
+        add_frac(nfy, N.ly, H6 * (dy + (T)2 * (e2y + e3y) + e4y) + H * S.d.ly());
+    }
     N.d = S.d;
     N.d.add_normalize(H6 * (k1x + (T)2 * (k2x + k3x) + k4x), H6 * (k1y + (T)2 * (k2y + k3y) + k4y));
     N.ci = S.ci;
     N.cj = S.cj;
     // f - 1 is exact for f in [1, 2); f + 1 for f in [-1, 0) rounds, so it goes
     // through the residual too
-    if (nfx >= (T)1) { N.ci += 1; nfx -= (T)1; } else if (nfx < (T)0) { N.ci -= 1; add_frac(nfx, N.lx, (T)1); }
-    if (nfy >= (T)1) { N.cj += 1; nfy -= (T)1; } else if (nfy < (T)0) { N.cj -= 1; add_frac(nfy, N.ly, (T)1); }
+    if (!in_unit(nfx, nfy)) {
+        if (nfx >= (T)1) { N.ci += 1; nfx -= (T)1; } else if (nfx < (T)0) { N.ci -= 1; add_frac(nfx, N.lx, (T)1); }
+        if (nfy >= (T)1) { N.cj += 1; nfy -= (T)1; } else if (nfy < (T)0) { N.cj -= 1; add_frac(nfy, N.ly, (T)1); }
+    }
     N.fx = nfx;
     N.fy = nfy;
 }
@@ -481,14 +516,21 @@ __device__ __forceinline__ void heun_step(CellT& C, const RayState<T>& S, T H, R
     T nfx = S.fx, nfy = S.fy;
     N.lx = S.lx;
     N.ly = S.ly;
-    add_frac(nfx, N.lx, Hh * (dx + e2x) + H * S.d.lx());
-    add_frac(nfy, N.ly, Hh * (dy + e2y) + H * S.d.ly());
+    if constexpr (sizeof(T) == 8) {
+        nfx += Hh * (dx + e2x);
+        nfy += Hh * (dy + e2y);
+    } else {
+        add_frac(nfx, N.lx, Hh * (dx + e2x) + H * S.d.lx());
+        add_frac(nfy, N.ly, Hh * (dy + e2y) + H * S.d.ly());
+    }
     N.d = S.d;
     N.d.add_normalize(Hh * (k1x + k2x), Hh * (k1y + k2y));
     N.ci = S.ci;
     N.cj = S.cj;
-    if (nfx >= (T)1) { N.ci += 1; nfx -= (T)1; } else if (nfx < (T)0) { N.ci -= 1; add_frac(nfx, N.lx, (T)1); }
-    if (nfy >= (T)1) { N.cj += 1; nfy -= (T)1; } else if (nfy < (T)0) { N.cj -= 1; add_frac(nfy, N.ly, (T)1); }
+    if (!in_unit(nfx, nfy)) {
+        if (nfx >= (T)1) { N.ci += 1; nfx -= (T)1; } else if (nfx < (T)0) { N.ci -= 1; add_frac(nfx, N.lx, (T)1); }
+        if (nfy >= (T)1) { N.cj += 1; nfy -= (T)1; } else if (nfy < (T)0) { N.cj -= 1; add_frac(nfy, N.ly, (T)1); }
+    }
     N.fx = nfx;
     N.fy = nfy;
 }
