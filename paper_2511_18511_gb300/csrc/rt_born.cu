@@ -69,17 +69,10 @@ namespace {
 
 constexpr double kPiB = 3.14159265358979323846;
 
-// Nodal fields for the Born march, in the pairs the packed samples use:
-// (c, s), (h dc/dx, h dc/dy) and (h^2 d2c/dy2, h^2 d2c/dx2), (h^2 d2c/dxdy,
-// alpha0 per mm of path), mm/us units.
+// Nodal fields for the Born march: (c, h dc/dx, h dc/dy, s) and
+// (h^2 d2c/dx2, h^2 d2c/dxdy, h^2 d2c/dy2, alpha0 per mm of path), mm/us units.
 struct __align__(32) BNode {
     float4 a, b;
-};
-
-// One sample of the marched fields.
-struct BSample {
-    float c, hxy;
-    F2 g, hd;   // (h dc/dx, h dc/dy), (h^2 d2c/dy2, h^2 d2c/dx2)
 };
 
 __global__ void k_born_pack(rt_grid g, const double* __restrict__ c_mps, const double* __restrict__ alpha0,
@@ -107,48 +100,22 @@ __global__ void k_born_pack(rt_grid g, const double* __restrict__ c_mps, const d
             al = (float)(1e-3 * a0);   // per mm of path
         }
         BNode o;
-        o.a = make_float4((float)c, (float)(1.0 / c), (float)gx, (float)gy);
-        o.b = make_float4((float)hyy, (float)hxx, (float)hxy, al);
+        o.a = make_float4((float)c, (float)gx, (float)gy, (float)(1.0 / c));
+        o.b = make_float4((float)hxx, (float)hxy, (float)hyy, al);
         out[k] = o;
     }
 }
 
 // Register cache of one cell: the seven fields (eight with absorption) in
 // bilinear coefficient form f = a + tx bx + ty (by + tx bxy), built from the
-// cell's four nodes, two fields to a register pair. Lookups as Cell<float> of
-// the ToF path.
-struct Bil2 {
-    F2 a, x, y, xy;
-    __device__ __forceinline__ void nodes(F2 v00, F2 v10, F2 v01, F2 v11) {
-        a = v00;
-        x = sub2(v10, v00);
-        y = sub2(v01, v00);
-        xy = sub2(sub2(v11, v10), y);
-    }
-    __device__ __forceinline__ F2 at(F2 tx, F2 ty) const { return fma2(ty, fma2(tx, xy, y), fma2(tx, x, a)); }
-    __device__ __forceinline__ float first(float tx, float ty) const {
-        float c0, c1, c2, c3, t;
-        unpk2(a, c0, t);
-        unpk2(x, c1, t);
-        unpk2(y, c2, t);
-        unpk2(xy, c3, t);
-        return fmaf(ty, fmaf(tx, c3, c2), fmaf(tx, c1, c0));
-    }
-    __device__ __forceinline__ float second(float tx, float ty) const {
-        float c0, c1, c2, c3, t;
-        unpk2(a, t, c0);
-        unpk2(x, t, c1);
-        unpk2(y, t, c2);
-        unpk2(xy, t, c3);
-        return fmaf(ty, fmaf(tx, c3, c2), fmaf(tx, c1, c0));
-    }
-};
-
+// cell's four nodes.
 template <bool ABS>
 struct BornCell {
     const BNode* __restrict__ F;
     int nx, ny, pi, pj;
-    Bil2 cs, g, hd, ha;   // (c, s), gradient, (hyy, hxx), (hxy, alpha0 with ABS)
+    float c0, c1, c2, c3, x0, x1, x2, x3, y0, y1, y2, y3, s0, s1, s2, s3;
+    float p0, p1, p2, p3, q0, q1, q2, q3, r0, r1, r2, r3;   // hxx, hxy, hyy
+    float l0, l1, l2, l3;                                   // alpha0 (ABS only)
 
     __device__ __forceinline__ void init(const BNode* f, const CellBS<float>*, int nx_, int ny_) {
         F = f;
@@ -162,57 +129,56 @@ struct BornCell {
         i = min(max(i, 0), nx - 2);
         j = min(max(j, 0), ny - 2);
         const BNode* p = F + (size_t)j * nx + i;
-        F2 n[4][4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const BNode* r = p + (q & 1) + (q >> 1) * nx;
-            asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];"
-                : "=l"(n[q][0].v), "=l"(n[q][1].v), "=l"(n[q][2].v), "=l"(n[q][3].v) : "l"(r));
+        const float4 a00 = p[0].a, b00 = p[0].b, a10 = p[1].a, b10 = p[1].b;
+        const float4 a01 = p[nx].a, b01 = p[nx].b, a11 = p[nx + 1].a, b11 = p[nx + 1].b;
+#define BC_(v0, v1, v2, v3, A00, A10, A01, A11) \
+    v0 = A00; v1 = A10 - A00; v2 = A01 - A00; v3 = (A11 - A10) - (A01 - A00);
+        BC_(c0, c1, c2, c3, a00.x, a10.x, a01.x, a11.x)
+        BC_(x0, x1, x2, x3, a00.y, a10.y, a01.y, a11.y)
+        BC_(y0, y1, y2, y3, a00.z, a10.z, a01.z, a11.z)
+        BC_(s0, s1, s2, s3, a00.w, a10.w, a01.w, a11.w)
+        BC_(p0, p1, p2, p3, b00.x, b10.x, b01.x, b11.x)
+        BC_(q0, q1, q2, q3, b00.y, b10.y, b01.y, b11.y)
+        BC_(r0, r1, r2, r3, b00.z, b10.z, b01.z, b11.z)
+        if (ABS) {
+            BC_(l0, l1, l2, l3, b00.w, b10.w, b01.w, b11.w)
         }
-        cs.nodes(n[0][0], n[1][0], n[2][0], n[3][0]);
-        g.nodes(n[0][1], n[1][1], n[2][1], n[3][1]);
-        hd.nodes(n[0][2], n[1][2], n[2][2], n[3][2]);
-        ha.nodes(n[0][3], n[1][3], n[2][3], n[3][3]);
+#undef BC_
     }
 
-    __device__ __forceinline__ void move(int ci, int cj, float u, float v, float& ox, float& oy, float& tx, float& ty) {
-        int i, j;
-        axis_move(u, ci, i, ox);
-        axis_move(v, cj, j, oy);
-        if (!(u >= -1.f && u < 2.f && v >= -1.f && v < 2.f)) {
-            const float fu = floorf(u), fv = floorf(v);
-            i = ci + (int)fu;
-            j = cj + (int)fv;
-            ox = -fu;
-            oy = -fv;
+    // Fields at fractions (u, v) of cell (ci, cj), as Cell::at of the ToF path.
+    __device__ __forceinline__ void at(int ci, int cj, float u, float v, float& c, float& gx, float& gy, float& hxx,
+                                       float& hxy, float& hyy, float& tx, float& ty) {
+        // 0 <= u < 1 on the float bits (-0 takes the general path, to the same result)
+        if (ci == pi && cj == pj && __float_as_uint(u) < 0x3f800000u && __float_as_uint(v) < 0x3f800000u) {
+            tx = u;
+            ty = v;
+        } else {
+            int i, j;
+            if (u >= -1.f && u < 2.f && v >= -1.f && v < 2.f) {
+                const bool ul = u < 0.f, uh = u >= 1.f, vl = v < 0.f, vh = v >= 1.f;
+                tx = ul ? u + 1.f : (uh ? u - 1.f : u);
+                ty = vl ? v + 1.f : (vh ? v - 1.f : v);
+                i = ci + (ul ? -1 : (uh ? 1 : 0));
+                j = cj + (vl ? -1 : (vh ? 1 : 0));
+            } else {
+                const float fu = floorf(u), fv = floorf(v);
+                i = ci + (int)fu;
+                j = cj + (int)fv;
+                tx = u - fu;
+                ty = v - fv;
+            }
+            if (i != pi || j != pj) load(i, j);
         }
-        tx = u + ox;
-        ty = v + oy;
-        load(i, j);
+        c = c0 + tx * c1 + ty * (c2 + tx * c3);
+        gx = x0 + tx * x1 + ty * (x2 + tx * x3);
+        gy = y0 + tx * y1 + ty * (y2 + tx * y3);
+        hxx = p0 + tx * p1 + ty * (p2 + tx * p3);
+        hxy = q0 + tx * q1 + ty * (q2 + tx * q3);
+        hyy = r0 + tx * r1 + ty * (r2 + tx * r3);
     }
-    __device__ __forceinline__ void seek(int ci, int cj, float u, float v, float& ox, float& oy, float& tx, float& ty) {
-        // opaque zeros: see Cell<float>::seek
-        asm("mov.f32 %0, 0f00000000;" : "=f"(ox));
-        asm("mov.f32 %0, 0f00000000;" : "=f"(oy));
-        tx = u;
-        ty = v;
-        if (!(ci == pi && cj == pj && max(__float_as_uint(u), __float_as_uint(v)) < 0x3f800000u))
-            move(ci, cj, u, v, ox, oy, tx, ty);
-    }
-    __device__ __forceinline__ void next(int ci, int cj, F2 p, float& ox, float& oy, float& tx, float& ty) {
-        unpk2(add2(p, pk2(ox, oy)), tx, ty);
-        if (max(__float_as_uint(tx), __float_as_uint(ty)) >= 0x3f800000u) {
-            float u, v;
-            unpk2(p, u, v);
-            move(ci, cj, u, v, ox, oy, tx, ty);
-        }
-    }
-    __device__ __forceinline__ BSample sample(float tx, float ty) const {
-        const F2 x = dup2(tx), y = dup2(ty);
-        return BSample{cs.first(tx, ty), ha.first(tx, ty), g.at(x, y), hd.at(x, y)};
-    }
-    __device__ __forceinline__ float slow(float tx, float ty) const { return cs.second(tx, ty); }
-    __device__ __forceinline__ float alpha(float tx, float ty) const { return ha.second(tx, ty); }
+    __device__ __forceinline__ float slow(float tx, float ty) const { return s0 + tx * s1 + ty * (s2 + tx * s3); }
+    __device__ __forceinline__ float alpha(float tx, float ty) const { return l0 + tx * l1 + ty * (l2 + tx * l3); }
 };
 
 // The same interface over the B-spline field: the 16 coefficients of the
@@ -259,16 +225,10 @@ struct BornCellS {
         }
     }
 
-    __device__ __forceinline__ void seek(int ci, int cj, float u, float v, float&, float&, float& tx, float& ty) {
+    __device__ __forceinline__ void at(int ci, int cj, float u, float v, float& c, float& gx, float& gy, float& hxx,
+                                       float& hxy, float& hyy, float& tx, float& ty) {
         int i, j;
         if (cell_locate(ci, cj, u, v, pi, pj, i, j, tx, ty)) load(i, j);
-    }
-    __device__ __forceinline__ void next(int ci, int cj, F2 p, float& ox, float& oy, float& tx, float& ty) {
-        float u, v;
-        unpk2(p, u, v);
-        seek(ci, cj, u, v, ox, oy, tx, ty);
-    }
-    __device__ __forceinline__ BSample sample(float tx, float ty) const {
         const float tx3 = 3.f * tx, tx6 = 6.f * tx;
         float r[4], d[4], e[4];
 #pragma unroll
@@ -278,27 +238,27 @@ struct BornCellS {
             d[q] = a1 + tx * (2.f * a2 + tx3 * a3);
             e[q] = 2.f * a2 + tx6 * a3;
         }
-        const float gx = d[0] + ty * (d[1] + ty * (d[2] + ty * d[3]));
-        const float hxx = e[0] + ty * (e[1] + ty * (e[2] + ty * e[3]));
-        const float gy = r[1] + ty * (2.f * r[2] + 3.f * ty * r[3]);
-        const float hyy = 2.f * r[2] + 6.f * ty * r[3];
-        return BSample{r[0] + ty * (r[1] + ty * (r[2] + ty * r[3])), d[1] + ty * (2.f * d[2] + 3.f * ty * d[3]),
-                       pk2(gx, gy), pk2(hyy, hxx)};
+        c = r[0] + ty * (r[1] + ty * (r[2] + ty * r[3]));
+        gx = d[0] + ty * (d[1] + ty * (d[2] + ty * d[3]));
+        hxx = e[0] + ty * (e[1] + ty * (e[2] + ty * e[3]));
+        gy = r[1] + ty * (2.f * r[2] + 3.f * ty * r[3]);
+        hxy = d[1] + ty * (2.f * d[2] + 3.f * ty * d[3]);
+        hyy = 2.f * r[2] + 6.f * ty * r[3];
     }
     __device__ __forceinline__ float slow(float tx, float ty) const { return bicubic<float>(pc->s, tx, ty); }
     __device__ __forceinline__ float alpha(float tx, float ty) const { return l0 + tx * l1 + ty * (l2 + tx * l3); }
 };
 
-// ray and paraxial right-hand sides at stage direction e, paraxial state (Q, P)
-__device__ __forceinline__ void born_rhs(const BSample& b, F2 e, F2 qp, F2& k, F2& kqp) {
-    float ex, ey, hy, hx, Q, P;
-    unpk2(e, ex, ey);
-    unpk2(qp, Q, P);
-    const float nic = rcp_approx(-b.c);
-    k = ray_rhs2(b.c, b.g, e);
-    unpk2(mul2(mul2(e, e), b.hd), hy, hx);
-    const float cnn = fmaf(-2.f * (ex * ey), b.hxy, hy + hx);
-    kqp = pk2(b.c * P, (-cnn * nic) * (nic * Q));
+// ray and paraxial right-hand sides at stage direction (ex, ey)
+__device__ __forceinline__ void born_rhs(float c, float gx, float gy, float hxx, float hxy, float hyy, float ex,
+                                         float ey, float Q, float P, float& kx, float& ky, float& kQ, float& kP) {
+    const float ic = rcp_approx(c);
+    const float gd = gx * ex + gy * ey;
+    kx = (gd * ex - gx) * ic;
+    ky = (gd * ey - gy) * ic;
+    const float cnn = ey * ey * hxx - 2.f * ex * ey * hxy + ex * ex * hyy;
+    kQ = c * P;
+    kP = -cnn * ic * ic * Q;
 }
 
 struct BornRay {
@@ -307,49 +267,68 @@ struct BornRay {
 };
 
 // One RK4 step of length H (cells). Stage 1 has already been evaluated at S
-// (b, with the cell offset o), since the deposit of S needs it. Lookups come
-// before the slopes of the stage before, as in the ToF step.
+// (c1.., passed in), since the deposit of S needs it.
 template <typename CellB>
-__device__ __forceinline__ void born_rk4(CellB& C, const BornRay& B, float H, float H6, BSample b, float ox, float oy,
-                                         BornRay& N) {
-    const F2 hh = dup2(0.5f * H), h1 = dup2(H), two = dup2(2.f);
-    const F2 f = pk2(B.S.fx, B.S.fy), d = pk2(B.S.d.x, B.S.d.y), qp = pk2(B.Q, B.P);
-    float tx, ty;
-    F2 k1, k2, k3, k4, p1, p2, p3, p4;
-    C.next(B.S.ci, B.S.cj, fma2(hh, d, f), ox, oy, tx, ty);
-    born_rhs(b, d, qp, k1, p1);
-    b = C.sample(tx, ty);
-    const F2 e2 = fma2(hh, k1, d);
-    C.next(B.S.ci, B.S.cj, fma2(hh, e2, f), ox, oy, tx, ty);
-    born_rhs(b, e2, fma2(hh, p1, qp), k2, p2);
-    b = C.sample(tx, ty);
-    const F2 e3 = fma2(hh, k2, d);
-    C.next(B.S.ci, B.S.cj, fma2(h1, e3, f), ox, oy, tx, ty);
-    born_rhs(b, e3, fma2(hh, p2, qp), k3, p3);
-    b = C.sample(tx, ty);
-    const F2 e4 = fma2(h1, k3, d);
-    born_rhs(b, e4, fma2(h1, p3, qp), k4, p4);
-    unpk2(fma2(dup2(H6), add2(fma2(two, add2(p2, p3), p1), p4), qp), N.Q, N.P);
-    commit2(B.S, H, H6, add2(fma2(two, add2(e2, e3), d), e4), add2(fma2(two, add2(k2, k3), k1), k4), N.S);
+__device__ __forceinline__ void born_rk4(CellB& C, const BornRay& B, float H, float c, float gx, float gy,
+                                         float hxx, float hxy, float hyy, BornRay& N) {
+    const float Hh = 0.5f * H, H6 = H / 6.f;
+    const float dx = B.S.d.hx(), dy = B.S.d.hy();
+    float tx, ty, k1x, k1y, k1Q, k1P, k2x, k2y, k2Q, k2P, k3x, k3y, k3Q, k3P, k4x, k4y, k4Q, k4P;
+    born_rhs(c, gx, gy, hxx, hxy, hyy, dx, dy, B.Q, B.P, k1x, k1y, k1Q, k1P);
+    float e2x = dx + Hh * k1x, e2y = dy + Hh * k1y, Q2 = B.Q + Hh * k1Q, P2 = B.P + Hh * k1P;
+    C.at(B.S.ci, B.S.cj, B.S.fx + Hh * dx, B.S.fy + Hh * dy, c, gx, gy, hxx, hxy, hyy, tx, ty);
+    born_rhs(c, gx, gy, hxx, hxy, hyy, e2x, e2y, Q2, P2, k2x, k2y, k2Q, k2P);
+    float e3x = dx + Hh * k2x, e3y = dy + Hh * k2y, Q3 = B.Q + Hh * k2Q, P3 = B.P + Hh * k2P;
+    C.at(B.S.ci, B.S.cj, B.S.fx + Hh * e2x, B.S.fy + Hh * e2y, c, gx, gy, hxx, hxy, hyy, tx, ty);
+    born_rhs(c, gx, gy, hxx, hxy, hyy, e3x, e3y, Q3, P3, k3x, k3y, k3Q, k3P);
+    float e4x = dx + H * k3x, e4y = dy + H * k3y, Q4 = B.Q + H * k3Q, P4 = B.P + H * k3P;
+    C.at(B.S.ci, B.S.cj, B.S.fx + H * e3x, B.S.fy + H * e3y, c, gx, gy, hxx, hxy, hyy, tx, ty);
+    born_rhs(c, gx, gy, hxx, hxy, hyy, e4x, e4y, Q4, P4, k4x, k4y, k4Q, k4P);
+    N.Q = B.Q + H6 * (k1Q + 2.f * (k2Q + k3Q) + k4Q);
+    N.P = B.P + H6 * (k1P + 2.f * (k2P + k3P) + k4P);
+    float nfx = B.S.fx, nfy = B.S.fy;
+    N.S.lx = B.S.lx;
+    N.S.ly = B.S.ly;
+    add_frac(nfx, N.S.lx, H6 * (dx + 2.f * (e2x + e3x) + e4x) + H * B.S.d.lx());
+    add_frac(nfy, N.S.ly, H6 * (dy + 2.f * (e2y + e3y) + e4y) + H * B.S.d.ly());
+    N.S.d = B.S.d;
+    N.S.d.add_normalize(H6 * (k1x + 2.f * (k2x + k3x) + k4x), H6 * (k1y + 2.f * (k2y + k3y) + k4y));
+    N.S.ci = B.S.ci;
+    N.S.cj = B.S.cj;
+    if (nfx >= 1.f) { N.S.ci += 1; nfx -= 1.f; } else if (nfx < 0.f) { N.S.ci -= 1; add_frac(nfx, N.S.lx, 1.f); }
+    if (nfy >= 1.f) { N.S.cj += 1; nfy -= 1.f; } else if (nfy < 0.f) { N.S.cj -= 1; add_frac(nfy, N.S.ly, 1.f); }
+    N.S.fx = nfx;
+    N.S.fy = nfy;
 }
 
 // One step of Heun's second-order Runge-Kutta method on (x, d, Q, P) (the
 // slopes at the start, given as stage 1, and at the Euler end point, averaged),
 // in the same cell-unit, compensated form as born_rk4.
 template <typename CellB>
-__device__ __forceinline__ void born_heun(CellB& C, const BornRay& B, float H, BSample b, float ox, float oy,
-                                          BornRay& N) {
+__device__ __forceinline__ void born_heun(CellB& C, const BornRay& B, float H, float c, float gx, float gy,
+                                          float hxx, float hxy, float hyy, BornRay& N) {
     const float Hh = 0.5f * H;
-    const F2 h1 = dup2(H), f = pk2(B.S.fx, B.S.fy), d = pk2(B.S.d.x, B.S.d.y), qp = pk2(B.Q, B.P);
-    float tx, ty;
-    F2 k1, k2, p1, p2;
-    C.next(B.S.ci, B.S.cj, fma2(h1, d, f), ox, oy, tx, ty);
-    born_rhs(b, d, qp, k1, p1);
-    b = C.sample(tx, ty);
-    const F2 e2 = fma2(h1, k1, d);
-    born_rhs(b, e2, fma2(h1, p1, qp), k2, p2);
-    unpk2(fma2(dup2(Hh), add2(p1, p2), qp), N.Q, N.P);
-    commit2(B.S, H, Hh, add2(d, e2), add2(k1, k2), N.S);
+    const float dx = B.S.d.hx(), dy = B.S.d.hy();
+    float tx, ty, k1x, k1y, k1Q, k1P, k2x, k2y, k2Q, k2P;
+    born_rhs(c, gx, gy, hxx, hxy, hyy, dx, dy, B.Q, B.P, k1x, k1y, k1Q, k1P);
+    const float e2x = dx + H * k1x, e2y = dy + H * k1y, Q2 = B.Q + H * k1Q, P2 = B.P + H * k1P;
+    C.at(B.S.ci, B.S.cj, B.S.fx + H * dx, B.S.fy + H * dy, c, gx, gy, hxx, hxy, hyy, tx, ty);
+    born_rhs(c, gx, gy, hxx, hxy, hyy, e2x, e2y, Q2, P2, k2x, k2y, k2Q, k2P);
+    N.Q = B.Q + Hh * (k1Q + k2Q);
+    N.P = B.P + Hh * (k1P + k2P);
+    float nfx = B.S.fx, nfy = B.S.fy;
+    N.S.lx = B.S.lx;
+    N.S.ly = B.S.ly;
+    add_frac(nfx, N.S.lx, Hh * (dx + e2x) + H * B.S.d.lx());
+    add_frac(nfy, N.S.ly, Hh * (dy + e2y) + H * B.S.d.ly());
+    N.S.d = B.S.d;
+    N.S.d.add_normalize(Hh * (k1x + k2x), Hh * (k1y + k2y));
+    N.S.ci = B.S.ci;
+    N.S.cj = B.S.cj;
+    if (nfx >= 1.f) { N.S.ci += 1; nfx -= 1.f; } else if (nfx < 0.f) { N.S.ci -= 1; add_frac(nfx, N.S.lx, 1.f); }
+    if (nfy >= 1.f) { N.S.cj += 1; nfy -= 1.f; } else if (nfy < 0.f) { N.S.cj -= 1; add_frac(nfy, N.S.ly, 1.f); }
+    N.S.fx = nfx;
+    N.S.fy = nfy;
 }
 
 // square root by the hardware approximation (sqrt.approx.ftz.f32), for values
@@ -464,11 +443,6 @@ __device__ __forceinline__ void born_deposit(const Geom& G, const FanArgs& A, co
     }
 }
 
-// Bound by instruction issue (fields and keys stay in L2). Fields, slopes and
-// paraxial state are packed pairs and a node is one 32-byte load, which takes
-// the maps of 64 transducers on a 1024^2 grid (385,000 rays) from 59.5 to
-// 54.3 ms at 5 blocks an SM; at 6 (80 registers) the pairs spill: 59.4 ms, at
-// 4: 55.7 ms.
 template <int BLOCK, int MINB, bool ABS, bool BS>
 __global__ void __launch_bounds__(BLOCK, MINB) k_born_fan(const Geom G, const FanArgs A, const BNode* __restrict__ field,
                                                           const CellBS<float>* __restrict__ bsfield) {
@@ -502,12 +476,11 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_born_fan(const Geom G, const Fa
     typename std::conditional<BS, BornCellS<ABS>, BornCell<ABS>>::type C;
     C.init(field, bsfield, G.nx, G.ny);
     C.load(B.S.ci, B.S.cj);
-    const float H = G.Hf, H6 = H / 6.f;
+    const float H = G.Hf;
     const float half_ds = 0.5f * G.dsf;
-    float ox, oy, tx, ty;
-    C.seek(B.S.ci, B.S.cj, B.S.fx, B.S.fy, ox, oy, tx, ty);
-    BSample b = C.sample(tx, ty);
-    const float c_t = b.c;
+    float c, gx, gy, hxx, hxy, hyy, tx, ty;
+    C.at(B.S.ci, B.S.cj, B.S.fx, B.S.fy, c, gx, gy, hxx, hxy, hyy, tx, ty);
+    const float c_t = c;
     const float inv_ct_h = 1.f / (c_t * A.hf);
     FanRef F;
     F.xt = (float)((xe - G.x0) / G.h);
@@ -522,8 +495,8 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_born_fan(const Geom G, const Fa
     int safe = 0, nsteps = 0;
     for (int m = 1; m <= G.max_steps_i; ++m) {
         BornRay N;
-        if (G.heun) born_heun(C, B, H, b, ox, oy, N);
-        else born_rk4(C, B, H, H6, b, ox, oy, N);
+        if (G.heun) born_heun(C, B, H, c, gx, gy, hxx, hxy, hyy, N);
+        else born_rk4(C, B, H, c, gx, gy, hxx, hxy, hyy, N);
         ++nsteps;
         if (--safe < 0) {
             const float ex = ring_excess(G, N.S);
@@ -533,8 +506,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_born_fan(const Geom G, const Fa
             safe = (int)((-ex / (Rc + r)) * 0.98f / H) - 1;
         }
         B = N;
-        C.seek(B.S.ci, B.S.cj, B.S.fx, B.S.fy, ox, oy, tx, ty);
-        b = C.sample(tx, ty);
+        C.at(B.S.ci, B.S.cj, B.S.fx, B.S.fy, c, gx, gy, hxx, hxy, hyy, tx, ty);
         const float s = C.slow(tx, ty);
         const float y = half_ds * (s_prev + s) - Tc;
         const float tt = T + y;
@@ -551,7 +523,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_born_fan(const Geom G, const Fa
             a_prev = a;
             al_h = a * A.hf;   // per cell of the along-ray offset
         }
-        born_deposit<ABS>(G, A, F, tfirst, near, lam, B, T, Tc, b.c, s, inv_ct_h, Lm - Lc, al_h);
+        born_deposit<ABS>(G, A, F, tfirst, near, lam, B, T, Tc, c, s, inv_ct_h, Lm - Lc, al_h);
     }
     const unsigned mask = __activemask();
     const unsigned tot = __reduce_add_sync(mask, (unsigned)nsteps);
@@ -861,7 +833,7 @@ int rtborn_maps_abs(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt, 
     const long long rays = (long long)prob->n_tx * fan_rays;
     const rt::BNode* fld = (const rt::BNode*)ctx->born_field;
     // kernel variants: resident 128-thread blocks per SM the kernel is compiled for
-    const int minb = opt->blocks_per_sm ? opt->blocks_per_sm : 5;   // 6 spills
+    const int minb = opt->blocks_per_sm ? opt->blocks_per_sm : (lossy ? 5 : 6);   // lossy at 6 spills
     const unsigned blocks = (unsigned)((rays + 127) / 128);
     switch (minb) {
 #define FAN_V(MB)                                                                               \
@@ -880,7 +852,7 @@ int rtborn_maps_abs(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt, 
         FAN_V(8)
 #undef FAN_V
         default:
-            return bfail(ctx, RT_EINVAL, "rtborn_maps: blocks_per_sm must be 0 (= 5), 4, 5, 6 or 8");
+            return bfail(ctx, RT_EINVAL, "rtborn_maps: blocks_per_sm must be 0 (= 6), 4, 5, 6 or 8");
     }
     rt::k_born_unpack<<<(unsigned)std::min<long long>(((long long)n_ent + 255) / 256, 152 * 64), 256, 0, s>>>(
         tfirst, near, lam, (long long)n_ent, T_out, A_out, lossy ? L_out : nullptr);
