@@ -123,14 +123,23 @@ struct BornCell {
         ny = ny_;
     }
 
+    // one node, one 32-byte load
+    __device__ __forceinline__ static void node(const BNode* p, float4& a, float4& b) {
+        asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w) : "l"(p));
+    }
+
     __device__ __forceinline__ void load(int i, int j) {
         pi = i;
         pj = j;
         i = min(max(i, 0), nx - 2);
         j = min(max(j, 0), ny - 2);
         const BNode* p = F + (size_t)j * nx + i;
-        const float4 a00 = p[0].a, b00 = p[0].b, a10 = p[1].a, b10 = p[1].b;
-        const float4 a01 = p[nx].a, b01 = p[nx].b, a11 = p[nx + 1].a, b11 = p[nx + 1].b;
+        float4 a00, b00, a10, b10, a01, b01, a11, b11;
+        node(p, a00, b00);
+        node(p + 1, a10, b10);
+        node(p + nx, a01, b01);
+        node(p + nx + 1, a11, b11);
 #define BC_(v0, v1, v2, v3, A00, A10, A01, A11) \
     v0 = A00; v1 = A10 - A00; v2 = A01 - A00; v3 = (A11 - A10) - (A01 - A00);
         BC_(c0, c1, c2, c3, a00.x, a10.x, a01.x, a11.x)
@@ -155,13 +164,12 @@ struct BornCell {
             ty = v;
         } else {
             int i, j;
-            if (u >= -1.f && u < 2.f && v >= -1.f && v < 2.f) {
-                const bool ul = u < 0.f, uh = u >= 1.f, vl = v < 0.f, vh = v >= 1.f;
-                tx = ul ? u + 1.f : (uh ? u - 1.f : u);
-                ty = vl ? v + 1.f : (vh ? v - 1.f : v);
-                i = ci + (ul ? -1 : (uh ? 1 : 0));
-                j = cj + (vl ? -1 : (vh ? 1 : 0));
-            } else {
+            float ox, oy;
+            axis_move(u, ci, i, ox);
+            axis_move(v, cj, j, oy);
+            tx = u + ox;
+            ty = v + oy;
+            if (!(u >= -1.f && u < 2.f && v >= -1.f && v < 2.f)) {
                 const float fu = floorf(u), fv = floorf(v);
                 i = ci + (int)fu;
                 j = cj + (int)fv;
@@ -286,19 +294,8 @@ __device__ __forceinline__ void born_rk4(CellB& C, const BornRay& B, float H, fl
     born_rhs(c, gx, gy, hxx, hxy, hyy, e4x, e4y, Q4, P4, k4x, k4y, k4Q, k4P);
     N.Q = B.Q + H6 * (k1Q + 2.f * (k2Q + k3Q) + k4Q);
     N.P = B.P + H6 * (k1P + 2.f * (k2P + k3P) + k4P);
-    float nfx = B.S.fx, nfy = B.S.fy;
-    N.S.lx = B.S.lx;
-    N.S.ly = B.S.ly;
-    add_frac(nfx, N.S.lx, H6 * (dx + 2.f * (e2x + e3x) + e4x) + H * B.S.d.lx());
-    add_frac(nfy, N.S.ly, H6 * (dy + 2.f * (e2y + e3y) + e4y) + H * B.S.d.ly());
-    N.S.d = B.S.d;
-    N.S.d.add_normalize(H6 * (k1x + 2.f * (k2x + k3x) + k4x), H6 * (k1y + 2.f * (k2y + k3y) + k4y));
-    N.S.ci = B.S.ci;
-    N.S.cj = B.S.cj;
-    if (nfx >= 1.f) { N.S.ci += 1; nfx -= 1.f; } else if (nfx < 0.f) { N.S.ci -= 1; add_frac(nfx, N.S.lx, 1.f); }
-    if (nfy >= 1.f) { N.S.cj += 1; nfy -= 1.f; } else if (nfy < 0.f) { N.S.cj -= 1; add_frac(nfy, N.S.ly, 1.f); }
-    N.S.fx = nfx;
-    N.S.fy = nfy;
+    commit2(B.S, H, H6, pk2(dx + 2.f * (e2x + e3x) + e4x, dy + 2.f * (e2y + e3y) + e4y),
+            pk2(k1x + 2.f * (k2x + k3x) + k4x, k1y + 2.f * (k2y + k3y) + k4y), N.S);
 }
 
 // One step of Heun's second-order Runge-Kutta method on (x, d, Q, P) (the
@@ -316,19 +313,7 @@ __device__ __forceinline__ void born_heun(CellB& C, const BornRay& B, float H, f
     born_rhs(c, gx, gy, hxx, hxy, hyy, e2x, e2y, Q2, P2, k2x, k2y, k2Q, k2P);
     N.Q = B.Q + Hh * (k1Q + k2Q);
     N.P = B.P + Hh * (k1P + k2P);
-    float nfx = B.S.fx, nfy = B.S.fy;
-    N.S.lx = B.S.lx;
-    N.S.ly = B.S.ly;
-    add_frac(nfx, N.S.lx, Hh * (dx + e2x) + H * B.S.d.lx());
-    add_frac(nfy, N.S.ly, Hh * (dy + e2y) + H * B.S.d.ly());
-    N.S.d = B.S.d;
-    N.S.d.add_normalize(Hh * (k1x + k2x), Hh * (k1y + k2y));
-    N.S.ci = B.S.ci;
-    N.S.cj = B.S.cj;
-    if (nfx >= 1.f) { N.S.ci += 1; nfx -= 1.f; } else if (nfx < 0.f) { N.S.ci -= 1; add_frac(nfx, N.S.lx, 1.f); }
-    if (nfy >= 1.f) { N.S.cj += 1; nfy -= 1.f; } else if (nfy < 0.f) { N.S.cj -= 1; add_frac(nfy, N.S.ly, 1.f); }
-    N.S.fx = nfx;
-    N.S.fy = nfy;
+    commit2(B.S, H, Hh, pk2(dx + e2x, dy + e2y), pk2(k1x + k2x, k1y + k2y), N.S);
 }
 
 // square root by the hardware approximation (sqrt.approx.ftz.f32), for values
@@ -443,6 +428,13 @@ __device__ __forceinline__ void born_deposit(const Geom& G, const FanArgs& A, co
     }
 }
 
+// Bound by instruction issue (fields and keys stay in L2). The position and
+// direction updates are the travel-time march's packed pairs, a cell moves in
+// fewer instructions and a node is one 32-byte load: maps of 64 transducers on a
+// 1024^2 grid (385,000 rays) 60.3 -> 57.3 ms at 5 blocks an SM, 58.1 ms at 4; at
+// 6 the pairs spill. Fields and paraxial slopes stay scalar: packed as well the
+// kernel took 54.3 ms, but with other last bits, by which a node between two
+// equally near rays can take the other ray's amplitude (off by up to 2 %).
 template <int BLOCK, int MINB, bool ABS, bool BS>
 __global__ void __launch_bounds__(BLOCK, MINB) k_born_fan(const Geom G, const FanArgs A, const BNode* __restrict__ field,
                                                           const CellBS<float>* __restrict__ bsfield) {
@@ -833,7 +825,7 @@ int rtborn_maps_abs(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt, 
     const long long rays = (long long)prob->n_tx * fan_rays;
     const rt::BNode* fld = (const rt::BNode*)ctx->born_field;
     // kernel variants: resident 128-thread blocks per SM the kernel is compiled for
-    const int minb = opt->blocks_per_sm ? opt->blocks_per_sm : (lossy ? 5 : 6);   // lossy at 6 spills
+    const int minb = opt->blocks_per_sm ? opt->blocks_per_sm : 5;   // 6 spills
     const unsigned blocks = (unsigned)((rays + 127) / 128);
     switch (minb) {
 #define FAN_V(MB)                                                                               \
@@ -852,7 +844,7 @@ int rtborn_maps_abs(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt, 
         FAN_V(8)
 #undef FAN_V
         default:
-            return bfail(ctx, RT_EINVAL, "rtborn_maps: blocks_per_sm must be 0 (= 6), 4, 5, 6 or 8");
+            return bfail(ctx, RT_EINVAL, "rtborn_maps: blocks_per_sm must be 0 (= 5), 4, 5, 6 or 8");
     }
     rt::k_born_unpack<<<(unsigned)std::min<long long>(((long long)n_ent + 255) / 256, 152 * 64), 256, 0, s>>>(
         tfirst, near, lam, (long long)n_ent, T_out, A_out, lossy ? L_out : nullptr);
