@@ -33,7 +33,7 @@
 //
 // Block roles (one block per SM): warp 0 allocates tensor memory and one of
 // its lanes issues the MMAs; warps 1-4 are the epilogue (warp w reads TMEM
-// lanes 32 (w mod 4) ...); warps 5-12 produce the A (and, for the apply, B)
+// lanes 32 (w mod 4) ...); warps 5-12 (5-20 in the apply) produce the A (and, for the apply, B)
 // stages; warp 13 (adjoint) issues the B copies. Two operand stages, two
 // accumulators (2 x 256 TMEM columns) so the epilogue of one accumulation
 // overlaps the next. Every wait is bounded (rt_tc.cuh): a stuck pipeline
@@ -64,7 +64,14 @@ constexpr uint32_t kStageBytes = 2 * kPlaneA + 2 * kPlaneB;   // A hi, A lo, B h
 constexpr int kStages = 2;
 constexpr int kEpiWarp0 = 1, kProdWarp0 = 5, kCopyWarp = 13;
 constexpr int kProdThreads = 256;
-constexpr int kApplyThreads = 13 * 32;
+// The apply is bound by its producers, which wait on map loads and chains of
+// special functions more than they issue: 16 warps forming 8 rows a thread in
+// place of 8 forming 16 take the 384-transducer, 4-frequency product at 1024^2
+// and its adjoint from 20.98 to 19.35 ms (the apply's share 13.8 -> 12.2).
+// Producer warps of the apply, and the A (and as many B) rows a thread of them
+// forms per stage.
+constexpr int kApplyProdWarps = 16, kApplyRows = kRows / (2 * kApplyProdWarps);
+constexpr int kApplyThreads = (kProdWarp0 + kApplyProdWarps) * 32;
 constexpr int kAdjThreads = 14 * 32;
 constexpr uint32_t kTmemCols = 512;
 constexpr int kBars = 9;   // full[2], empty[2], acc_full[2], acc_empty[2], drain
@@ -213,7 +220,7 @@ template <bool LOSSY>
 __global__ void __launch_bounds__(kApplyThreads, 1) k_born_apply_tc(const __grid_constant__ TCArgs a) {
     extern __shared__ uint8_t smem_raw[];
     const Smem S = carve(smem_raw);
-    setup(S, kProdThreads / 32);
+    setup(S, kApplyProdWarps);
     const uint32_t tmem = *S.tslot;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int U = a.n_freq * a.n_tiles;
@@ -275,11 +282,11 @@ __global__ void __launch_bounds__(kApplyThreads, 1) k_born_apply_tc(const __grid
     } else if (warp >= kProdWarp0) {
         // a half-warp covers the 16 nodes of one K-tile for one transducer row,
         // so every map load of a warp reads two rows x 64 contiguous bytes.
-        // Rows of this thread: A rows tA + 16 i and B rows tB + 16 i (i < 8).
-        // All 16 (or 24) map values of a stage are loaded before any is used,
-        // and those of the next stage while this one is formed.
+        // Rows of this thread: A rows tA + kStep i and B rows tB + kStep i
+        // (i < kApplyRows). All its map values of a stage are loaded before any
+        // is used, and those of the next stage while this one is formed.
         const int pw = warp - kProdWarp0, j = lane & 15, sub = lane >> 4;
-        constexpr int NL = LOSSY ? 16 : 1;
+        constexpr int kStep = 2 * kApplyProdWarps, NM = 2 * kApplyRows, NL = LOSSY ? NM : 1;
         uint32_t q = 0;
         for (long long it = blockIdx.x; it < a.n_items; it += gridDim.x) {
             const int c = (int)(it / U), u = (int)(it % U);
@@ -289,7 +296,7 @@ __global__ void __launch_bounds__(kApplyThreads, 1) k_born_apply_tc(const __grid
             const BornFreq& fq = a.fq[f];
             const int tA = bi * kRows + 2 * pw + sub, tB = bj * kRows + 2 * pw + sub;
             const int kt0 = c * a.chunk, kt1 = min(kt0 + a.chunk, a.nk);
-            float Tn[16], An[16], Ln[NL], wn;
+            float Tn[NM], An[NM], Ln[NL], wn;
             bool pvn;
             auto load = [&](int kt) {
                 const int p = kt * 16 + j;
@@ -297,8 +304,8 @@ __global__ void __launch_bounds__(kApplyThreads, 1) k_born_apply_tc(const __grid
                 const int k = a.idx[p];
                 wn = a.dc[k];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int t = (i < 8 ? tA : tB) + 16 * (i & 7);
+                for (int i = 0; i < NM; ++i) {
+                    const int t = (i < kApplyRows ? tA : tB) + kStep * (i % kApplyRows);
                     const bool v = pvn && t < a.n_tx;
                     const size_t o = (size_t)(v ? t : 0) * (size_t)a.nn + k;
                     Tn[i] = v ? a.T[o] : __uint_as_float(0x7f800000u);
@@ -309,9 +316,9 @@ __global__ void __launch_bounds__(kApplyThreads, 1) k_born_apply_tc(const __grid
             load(kt0);
             bool ok = true;
             for (int kt = kt0; kt < kt1; ++kt, ++q) {
-                float Tc[16], Ac[16], Lc[NL];
+                float Tc[NM], Ac[NM], Lc[NL];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
+                for (int i = 0; i < NM; ++i) {
                     Tc[i] = Tn[i];
                     Ac[i] = An[i];
                     if (LOSSY) Lc[i & (NL - 1)] = Ln[i & (NL - 1)];
@@ -324,11 +331,11 @@ __global__ void __launch_bounds__(kApplyThreads, 1) k_born_apply_tc(const __grid
                 const uint32_t sb = S.base + st * kStageBytes;
                 const uint32_t cofs = (uint32_t)(j & 1) * 8u;
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int m = 2 * pw + sub + 16 * (i & 7);
+                for (int i = 0; i < NM; ++i) {
+                    const int m = 2 * pw + sub + kStep * (i % kApplyRows);
                     const float2 E = efield<LOSSY>(Tc[i], Ac[i], LOSSY ? Lc[i & (NL - 1)] : 0.f, fq);
                     const uint32_t off = swz(m, j >> 1) + cofs;
-                    if (i < 8) {
+                    if (i < kApplyRows) {
                         const float hr = to_tf32(E.x), hi = to_tf32(E.y);
                         st_shared_v2(sb + off, hr, hi);
                         st_shared_v2(sb + kPlaneA + off, to_tf32(E.x - hr), to_tf32(E.y - hi));
