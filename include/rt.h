@@ -386,9 +386,9 @@ typedef struct {
 /*
  * rt_batch_run — rt_link plus, for instances with tof_ref, the adjoint of the
  * L2 misfit (rt_tof_adjoint with g_tof = T), for n_inst problems of different
- * grids and rings in ONE persistent launch over all their pairs (longest rings
- * first, longest chords first within a ring). Each pair is linked (paper
- * Sec. 3.4) and then, in a second launch, retraced with its adjoint weight
+ * grids and rings: their fans in one launch, then one persistent launch that
+ * links all their pairs (longest rings first, longest chords first within a
+ * ring; paper Sec. 3.4), then one that retraces them with the adjoint weight
  * T - T_ref (Sec. 3.1.1).
  *   inst   HOST array of n_inst descriptors (read during the call).
  * Every per-instance output is as for rt_link / rt_tof_adjoint; status counts

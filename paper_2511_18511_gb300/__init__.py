@@ -427,7 +427,7 @@ def rt_batch_run(instances, ds: float, tol: float = 1e-4, max_iter: int = 30, pr
                  blocks_per_sm: int = 0, ctx: Optional[Context] = None, stream=None,
                  reset_angles: bool = True, integrator: str = "rk4"):
     """Link (and, where tof_ref is set, adjoint-scatter) every pair of every
-    instance in one persistent launch. reset_angles=True starts cold (NaN)."""
+    instance, all in the same launches. reset_angles=True starts cold (NaN)."""
     ctx = ctx or default_context(instances[0].prob.c.device.index)
     if reset_angles:
         for b in instances:
