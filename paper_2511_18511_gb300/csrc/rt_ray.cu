@@ -269,18 +269,22 @@ __global__ void __launch_bounds__(kBlock) k_fan_batch(const __grid_constant__ Fa
 // linking state when a trace ends, so lanes never wait for other lanes' pairs
 // (a lane whose trace ends early in an iteration idles for the rest of it).
 // The iteration's bookkeeping (queue fetch, reconvergence of the warp) cost a
-// lone lane about 85 ns per step at one step per iteration: 537 against 363 ns
-// per RK4 step for the plain traced-ray kernel; at 16 steps it is 428 ns.
+// lone lane about 85 ns per step at one step per iteration with the scalar
+// step: 537 against 363 ns per RK4 step for the plain traced-ray kernel (266 ns
+// now); at 16 steps it was 428 ns.
 // Resident blocks per SM the link kernel is compiled for. The recording
 // variant, which keeps a run accumulator per lane, runs 4 blocks (128
-// registers): 53.0 against 54.5 ms at 5 on the cold breast workload. The plain
-// FP32 link stays at 6 (80 registers): at 5 its cold link was no faster and
-// its warm start (one trace per pair, throughput-bound) slower.
+// registers): the cold breast workload takes 45.7 ms, 47.8 at 5, and a warm
+// link of 41,006 pairs with its gradient 22.2 against 27.6 ms (the full warm
+// breast link 22.2 against 20.9). The plain FP32 link stays at 6 (80
+// registers): at 5 its cold link was no faster (39.1 to 40.4 ms) and its warm
+// start (one trace per pair, bound by issue) 17.5 against 15.9 ms.
 template <typename T, int I, bool REC> struct LinkBlocks { static constexpr int v = Occ<T, I>::blocks; };
 template <typename T, int I> struct LinkBlocks<T, I, true> { static constexpr int v = 4; };
 
-// RK4 steps per loop iteration of k_link (measured on the breast workload:
-// 1 -> 60.6 ms, 4 -> 55.1, 8 -> 54.5, 16 -> 53.6 for the recording link)
+// RK4 steps per loop iteration of k_link (measured on the breast workload with
+// the scalar step: 1 -> 60.6 ms, 4 -> 55.1, 8 -> 54.5, 16 -> 53.6 for the
+// recording link, 45.5 now; unrolling the 16 by two: 46.9)
 constexpr int kLinkSteps = 16;
 
 template <typename T, int I, bool REC, bool ROUNDS = false>
