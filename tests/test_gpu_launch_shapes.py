@@ -115,3 +115,29 @@ def test_batch_of_several_is_each_alone(rt):
         for name in ("theta", "tof", "hit", "status", "iters"):
             assert torch.equal(getattr(b, name), getattr(alone, name))
         assert ((b.g_c - alone.g_c).abs() <= 1e-11 * alone.g_c.abs()).all()
+
+
+# Nodes, frequencies and transducers at which the apply's items fill the SMs in
+# chunks of 4 to 16 K-tiles, whole and ragged.
+@pytest.mark.parametrize("n", [40, 97, 128])
+@pytest.mark.parametrize("n_tx,n_freq", [(5, 1), (64, 8), (130, 3)])
+def test_born_apply_chunks(rt, n, n_tx, n_freq):
+    """The tensor-core product against the FP32 SIMT product of the same maps:
+    both sum at most 12,900 nodes, whose FP32 roundings (2^-24 each, adding like
+    a random walk) and the split's 2^-21 per product stay below 2e-5."""
+    from paper_2511_18511_gb300 import phantoms as P
+    h = 0.5
+    R = 0.45 * n * h
+    x = (torch.arange(n, dtype=torch.float64, device="cuda") - (n - 1) / 2) * h
+    inside = x[None, :] ** 2 + x[:, None] ** 2 < R * R
+    tx = torch.as_tensor(P.ring(n_tx, R), device="cuda")
+    r = torch.sqrt((x[None, None, :] - tx[:, 0, None, None]) ** 2 + (x[None, :, None] - tx[:, 1, None, None]) ** 2)
+    T = torch.where(inside, r / 1.5, torch.inf).float().contiguous()
+    A = torch.where(inside, torch.rsqrt(r.clamp(min=h)), 0.0).float().contiguous()
+    maps = rt.BornMaps(P.Grid(n, n, h), R, T, A)
+    g = torch.Generator().manual_seed(n + n_tx)
+    dc = torch.where(inside, torch.randn(n, n, generator=g, dtype=torch.float64).cuda(), 0.0).float().contiguous()
+    f = [0.4 + 0.1 * k for k in range(n_freq)]
+    a = rt.rtborn_apply(maps, f, dc, gemm="tf32x3").to(torch.complex128)
+    b = rt.rtborn_apply(maps, f, dc, gemm="fp32").to(torch.complex128)
+    assert float((a - b).abs().pow(2).sum().sqrt()) <= 2e-5 * float(b.abs().pow(2).sum().sqrt())
