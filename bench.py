@@ -197,14 +197,14 @@ def batch_leg(args, peaks, steps: int = 3, warmup: int = 3, fp64_every: int = 4)
                          "frac": achieved / fp32,
                          "traffic": (_traffic(os.path.join(ROOT, "profiles", "batch_traffic.json"), BATCH_HASH_FILES)
                                      if tuple(best) == BATCH_PROFILE_VARIANT else None),
-                         "kernel": "graph replay (pack + fan + k_batch + finish)", "flop_per_rk4_step": FLOP_PER_STEP,
+                         "kernel": "graph replay (pack + k_fan_batch + k_batch + k_batch_adjoint + finish)", "flop_per_rk4_step": FLOP_PER_STEP,
                          "rk4_steps_per_launch": counts[7], "peak_basis": "measured FP32 FMA rate (rt_peak_fma)"},
             "link": {"all_linked": ok, "status_counts": counts[:7]},
             "fp32c_vs_fp64": {"instances": len(sub), "pairs": n_sub,
                               "fp32c": {"value": n_sub / (ms_sub32 / 1e3), "ms": ms_sub32},
                               "fp64": {"value": n_sub / (ms_sub64 / 1e3), "ms": ms_sub64},
                               "speedup_fp32c_over_fp64": ms_sub64 / ms_sub32},
-            "gpu_launches_per_step": 3 * len(insts) + 2}
+            "gpu_launches_per_step": 2 * len(insts) + 4}
 
 
 def run_batch(args):
