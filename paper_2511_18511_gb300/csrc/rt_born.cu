@@ -431,8 +431,9 @@ __device__ __forceinline__ void born_deposit(const Geom& G, const FanArgs& A, co
 // Bound by instruction issue (fields and keys stay in L2). The position and
 // direction updates are the travel-time march's packed pairs, a cell moves in
 // fewer instructions and a node is one 32-byte load: maps of 64 transducers on a
-// 1024^2 grid (385,000 rays) 60.3 -> 57.3 ms on one board and 58.8 -> 58.0 ms on
-// another at 5 blocks an SM, 58.1 ms at 4 on the first; at 6 the pairs spill. Fields and paraxial slopes stay scalar: packed as well the
+// 1024^2 grid (385,000 rays) 60.3 -> 57.3 ms on one board, 58.4 -> 56.8 and
+// 58.8 -> 58.0 ms on others at 5 blocks an SM, 58.1 ms at 4 on the first; at 6
+// the pairs spill. Fields and paraxial slopes stay scalar: packed as well the
 // kernel took 54.3 ms, but with other last bits, by which a node between two
 // equally near rays can take the other ray's amplitude (off by up to 2 %).
 template <int BLOCK, int MINB, bool ABS, bool BS>

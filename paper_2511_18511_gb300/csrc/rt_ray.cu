@@ -521,7 +521,8 @@ static void link_impl(const Geom& G, const void* field, double tol, int max_iter
     const int pb = persistent_blocks(k_link<T, I, REC, ROUNDS>, slot);
     const long long warps = std::min<long long>((long long)pb * (kLinkBlock / 32), (long long)sm_count() * kLinkSpreadWarps);
     const long long pairs = G.n_pairs;   // an upper bound of the pairs a rounds launch resumes
-    const int lanes = (int)std::min<long long>(32, std::max<long long>(sizeof(T) == 8 ? kMinLanes64 : 1, (pairs + warps - 1) / warps));
+    const long long least = sizeof(T) == 8 ? kMinLanes64 : 1;
+    const int lanes = (int)std::min<long long>(32, std::max<long long>(least, (pairs + warps - 1) / warps));
     const long long per_block = (long long)lanes * (kLinkBlock / 32);
     const int nb = (int)std::min<long long>(pb, (pairs + per_block - 1) / per_block);
     k_link<T, I, REC, ROUNDS><<<nb, kLinkBlock, 0, s>>>(G, (const typename Samp<T, I>::Field*)field, tol, max_iter,
