@@ -268,6 +268,51 @@ def rt_tof_adjoint(prob: Problem, theta: torch.Tensor, g_tof: torch.Tensor, ds: 
 
 
 RECORD_BYTES = 16 << 30   # most memory rt_path_matrix takes for the recorded visits
+RECORD_FREE_ASK = 1 << 30   # a record above this takes at most a quarter of the device's free memory
+
+
+def _record_fits(size: int, dev) -> bool:
+    """Whether rt_path_matrix may take `size` bytes for its record. The block
+    stays in torch's cache afterwards, where the library's own allocations do
+    not find it: a large one leaves most of what is free."""
+    if not 0 < size <= RECORD_BYTES:
+        return False
+    if size <= RECORD_FREE_ASK:
+        return True
+    free = torch.cuda.mem_get_info(dev)[0] + torch.cuda.memory_reserved(dev) - torch.cuda.memory_allocated(dev)
+    return size <= free // 4
+
+
+def _path_matrix_recorded(ctx, ps, o, th, row_ptr, cap: int, size: int, stream):
+    """The matrix from one trace per ray, whose cell visits are kept while it is
+    laid out (a third of the time of counting, counting and filling by three
+    traces). The visits take about as much memory as the matrix. None if a row is
+    longer than its record or memory is short; the record is then given back,
+    to the library's allocations too."""
+    dev = row_ptr.device
+    nnz = C.c_int64(0)
+    try:
+        runs = torch.empty(size, dtype=torch.uint8, device=dev)
+        rec = _L.RtRows(runs.data_ptr(), None, cap)
+        rc = ctx.lib.rt_path_record(ctx.h, C.byref(ps), C.byref(o), _ptr(th), C.byref(rec), _ptr(row_ptr),
+                                    C.byref(nnz), _stream(stream))
+        if rc == _L.RT_OK:
+            col = torch.empty(max(nnz.value, 1), dtype=torch.int32, device=dev)
+            val = torch.empty(max(nnz.value, 1), dtype=torch.float64, device=dev)
+            _L.check(ctx.h, ctx.lib.rt_path_expand(ctx.h, C.byref(ps), C.byref(rec), _ptr(row_ptr), _ptr(col),
+                                                   _ptr(val), _stream(stream)))
+            if stream is not None:
+                runs.record_stream(stream)   # freed below, still read there
+            return row_ptr, col[: nnz.value], val[: nnz.value]
+        if rc != _L.RT_ENOMEM:
+            _L.check(ctx.h, rc)
+        short = nnz.value == 0               # the library's workspace, not a long row
+    except torch.OutOfMemoryError:
+        short = True
+    runs = col = val = None
+    if short:
+        torch.cuda.empty_cache()
+    return None
 
 
 def rt_path_matrix(prob: Problem, theta: torch.Tensor, ds: float, precision: str = "fp32c",
@@ -283,30 +328,12 @@ def rt_path_matrix(prob: Problem, theta: torch.Tensor, ds: float, precision: str
     ps = prob.struct(c)
     o = _opts(ds, precision=precision, integrator=integrator, interpolator=interpolator)
     th = theta.contiguous()
-    # one trace per ray: its cell visits are kept while the matrix is laid out
-    # (a third of the time of counting, counting and filling by three traces).
-    # The visits take about as much memory as the matrix, hence the limit.
     cap = ctx.lib.rt_rows_cap(C.byref(ps))
     size = prob.n_pairs * cap * _L.RUN_BYTES
-    if precision == "fp32c" and interpolator == "bilinear" and 0 < size <= RECORD_BYTES:
-        try:
-            runs = torch.empty(size, dtype=torch.uint8, device=dev)
-        except torch.OutOfMemoryError:
-            runs = None
-        if runs is not None:
-            rec = _L.RtRows(runs.data_ptr(), None, cap)
-            rc = ctx.lib.rt_path_record(ctx.h, C.byref(ps), C.byref(o), _ptr(th), C.byref(rec), _ptr(row_ptr),
-                                        C.byref(nnz), _stream(stream))
-            if rc == _L.RT_OK:
-                col = torch.empty(max(nnz.value, 1), dtype=torch.int32, device=dev)
-                val = torch.empty(max(nnz.value, 1), dtype=torch.float64, device=dev)
-                _L.check(ctx.h, ctx.lib.rt_path_expand(ctx.h, C.byref(ps), C.byref(rec), _ptr(row_ptr), _ptr(col),
-                                                       _ptr(val), _stream(stream)))
-                if stream is not None:
-                    runs.record_stream(stream)   # freed below, still read there
-                return row_ptr, col[: nnz.value], val[: nnz.value]
-            if rc != _L.RT_ENOMEM:
-                _L.check(ctx.h, rc)
+    if precision == "fp32c" and interpolator == "bilinear" and _record_fits(size, dev):
+        got = _path_matrix_recorded(ctx, ps, o, th, row_ptr, cap, size, stream)
+        if got is not None:
+            return got
     rc = ctx.lib.rt_path_matrix(ctx.h, C.byref(ps), C.byref(o), _ptr(th), _ptr(row_ptr), None, None, 0,
                                 C.byref(nnz), _stream(stream))
     if rc not in (_L.RT_OK, _L.RT_ENOMEM):

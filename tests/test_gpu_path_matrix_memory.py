@@ -1,0 +1,117 @@
+"""rt_path_matrix where memory is short: the matrix from one trace keeps a
+record of about the matrix's size, and a call that has room for the matrix
+alone gives the same matrix by counting and filling."""
+import weakref
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rt():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2511_18511_gb300 as m
+    return m
+
+
+@pytest.fixture(scope="module")
+def case(rt):
+    from paper_2511_18511_gb300 import phantoms as P
+    nx, h, n_tx = 101, 0.5, 96
+    R = 0.42 * nx * h
+    x = (np.arange(nx) - (nx - 1) / 2) * h
+    c = 1500.0 * (1.0 + 0.03 * np.cos(x / 5.0)[None, :] * np.cos(x / 7.0)[:, None])
+    prob = rt.Problem.create(P.Grid(nx, nx, h), c, P.ring(n_tx, R), R)
+    e = torch.arange(n_tx, device="cuda").repeat_interleave(n_tx - 1)
+    r = torch.arange(n_tx - 1, device="cuda").repeat(n_tx)
+    d = prob.tx[r + (r >= e).long()] - prob.tx[e]
+    theta = torch.atan2(d[:, 1], d[:, 0]).contiguous()
+    ds = 0.1 * h
+    return prob, theta, ds, rt.rt_path_matrix(prob, theta, ds)
+
+
+class _Record:
+    """torch.empty that notes the record's block and can refuse later ones."""
+
+    def __init__(self, refuse=None):
+        self.real, self.refuse, self.ref, self.size = torch.empty, refuse, lambda: None, 0
+
+    def __call__(self, *a, **k):
+        if k.get("dtype") is self.refuse and self.ref() is not None:
+            raise torch.OutOfMemoryError("no room beside the record")
+        t = self.real(*a, **k)
+        if k.get("dtype") is torch.uint8:
+            self.ref, self.size = weakref.ref(t), t.numel()
+        return t
+
+
+class _Ctx:
+    """A context whose library calls can be replaced."""
+
+    def __init__(self, ctx, **calls):
+        self.h, self.lib = ctx.h, type("Lib", (), {"__getattr__": lambda _, n: calls.get(n) or getattr(ctx.lib, n)})()
+
+
+def _same(got, want):
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("refuse", [torch.int32, torch.float64])
+def test_no_room_for_the_matrix_beside_the_record(rt, case, refuse, monkeypatch):
+    prob, theta, ds, want = case
+    empty = _Record(refuse)
+    monkeypatch.setattr(torch, "empty", empty)
+    _same(rt.rt_path_matrix(prob, theta, ds), want)
+    assert empty.size > 0                          # the record was tried
+
+
+def test_no_room_for_the_library_beside_the_record(rt, case, monkeypatch):
+    """The record's block goes back to the device before the library is called again."""
+    from paper_2511_18511_gb300 import _lib as L
+    prob, theta, ds, want = case
+    ctx = rt.default_context(prob.c.device.index)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.memory_reserved()
+    empty = _Record()
+    monkeypatch.setattr(torch, "empty", empty)
+    reserved = []
+
+    def matrix(*a):
+        reserved.append(torch.cuda.memory_reserved())
+        return ctx.lib.rt_path_matrix(*a)
+
+    _same(rt.rt_path_matrix(prob, theta, ds, ctx=_Ctx(ctx, rt_path_record=lambda *a: L.RT_ENOMEM,
+                                                      rt_path_matrix=matrix)), want)
+    assert empty.size > 20 << 20 and empty.ref() is None
+    assert reserved[0] < before + empty.size
+
+
+def test_large_record_leaves_most_of_the_free_memory(rt, case, monkeypatch):
+    from paper_2511_18511_gb300 import _lib as L
+    prob, theta, ds, want = case
+    ctx = rt.default_context(prob.c.device.index)
+    calls = []
+
+    def record(*a):
+        calls.append(1)
+        return ctx.lib.rt_path_record(*a)
+
+    monkeypatch.setattr(rt, "RECORD_FREE_ASK", 0, raising=False)
+    cap = ctx.lib.rt_rows_cap(prob.struct())
+    size = prob.n_pairs * cap * L.RUN_BYTES
+    for free, taken in ((4 * size, 1), (2 * size, 0)):
+        # nothing of torch's cache counts here
+        monkeypatch.setattr(torch.cuda, "mem_get_info", lambda dev=None: (free, 1 << 40))
+        monkeypatch.setattr(torch.cuda, "memory_reserved", lambda dev=None: 0)
+        monkeypatch.setattr(torch.cuda, "memory_allocated", lambda dev=None: 0)
+        calls.clear()
+        _same(rt.rt_path_matrix(prob, theta, ds, ctx=_Ctx(ctx, rt_path_record=record)), want)
+        assert len(calls) == taken
