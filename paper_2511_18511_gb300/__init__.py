@@ -292,7 +292,13 @@ def _path_matrix_recorded(ctx, ps, o, th, row_ptr, cap: int, size: int, stream):
     dev = row_ptr.device
     nnz = C.c_int64(0)
     try:
-        runs = torch.empty(size, dtype=torch.uint8, device=dev)
+        # from the pool of the stream that writes and reads it: a block of another
+        # stream's pool may still be in use there, and would go back there too early
+        own = stream                         # None: the current one
+        if stream is not None and not isinstance(stream, torch.cuda.Stream):
+            own = torch.cuda.ExternalStream(stream.cuda_stream, device=dev)
+        with torch.cuda.stream(own):
+            runs = torch.empty(size, dtype=torch.uint8, device=dev)
         rec = _L.RtRows(runs.data_ptr(), None, cap)
         rc = ctx.lib.rt_path_record(ctx.h, C.byref(ps), C.byref(o), _ptr(th), C.byref(rec), _ptr(row_ptr),
                                     C.byref(nnz), _stream(stream))
@@ -301,8 +307,6 @@ def _path_matrix_recorded(ctx, ps, o, th, row_ptr, cap: int, size: int, stream):
             val = torch.empty(max(nnz.value, 1), dtype=torch.float64, device=dev)
             _L.check(ctx.h, ctx.lib.rt_path_expand(ctx.h, C.byref(ps), C.byref(rec), _ptr(row_ptr), _ptr(col),
                                                    _ptr(val), _stream(stream)))
-            if stream is not None:
-                runs.record_stream(stream)   # freed below, still read there
             return row_ptr, col[: nnz.value], val[: nnz.value]
         if rc != _L.RT_ENOMEM:
             _L.check(ctx.h, rc)

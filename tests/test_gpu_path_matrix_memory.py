@@ -1,6 +1,7 @@
 """rt_path_matrix where memory is short: the matrix from one trace keeps a
 record of about the matrix's size, and a call that has room for the matrix
 alone gives the same matrix by counting and filling."""
+import types
 import weakref
 
 import numpy as np
@@ -41,14 +42,14 @@ class _Record:
     """torch.empty that notes the record's block and can refuse later ones."""
 
     def __init__(self, refuse=None):
-        self.real, self.refuse, self.ref, self.size = torch.empty, refuse, lambda: None, 0
+        self.real, self.refuse, self.ref, self.size, self.stream = torch.empty, refuse, lambda: None, 0, None
 
     def __call__(self, *a, **k):
         if k.get("dtype") is self.refuse and self.ref() is not None:
             raise torch.OutOfMemoryError("no room beside the record")
         t = self.real(*a, **k)
         if k.get("dtype") is torch.uint8:
-            self.ref, self.size = weakref.ref(t), t.numel()
+            self.ref, self.size, self.stream = weakref.ref(t), t.numel(), torch.cuda.current_stream()
         return t
 
 
@@ -115,3 +116,17 @@ def test_large_record_leaves_most_of_the_free_memory(rt, case, monkeypatch):
         calls.clear()
         _same(rt.rt_path_matrix(prob, theta, ds, ctx=_Ctx(ctx, rt_path_record=record)), want)
         assert len(calls) == taken
+
+
+@pytest.mark.parametrize("handle", [lambda s: s, lambda s: types.SimpleNamespace(cuda_stream=s.cuda_stream)])
+def test_record_belongs_to_the_stream_that_uses_it(rt, case, handle, monkeypatch):
+    """The allocator orders a block's uses on the stream it was taken on only."""
+    prob, theta, ds, want = case
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    empty = _Record()
+    monkeypatch.setattr(torch, "empty", empty)
+    got = rt.rt_path_matrix(prob, theta, ds, stream=handle(side))
+    assert empty.stream.cuda_stream == side.cuda_stream != torch.cuda.current_stream().cuda_stream
+    side.synchronize()
+    _same(got, want)
