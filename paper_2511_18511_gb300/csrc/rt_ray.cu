@@ -982,7 +982,10 @@ __global__ void __launch_bounds__(kBlock) k_rows_record(Geom G, const CellCoef<f
 }
 
 // The entries of the recorded rows, a warp per pair, a lane per visit: 16-byte
-// column and value stores (rows start at multiples of four entries).
+// column and value stores (rows start at multiples of four entries). A row may
+// be longer than its record (rt_path_record reports that): its entries beyond
+// are column 0 with value NaN, so nothing is read past the record and no product
+// with such a matrix passes for a result.
 __global__ void __launch_bounds__(kBlock) k_rows_expand(int n_pairs, int nx, const int64_t* __restrict__ row_ptr,
                                                         RowRec rec, int32_t* __restrict__ col, double* __restrict__ val,
                                                         int vec) {
@@ -992,6 +995,15 @@ __global__ void __launch_bounds__(kBlock) k_rows_expand(int n_pairs, int nx, con
     const int n = (int)((row_ptr[k + 1] - b) >> 2);
     const rt_run* row = rec.runs + (size_t)k * rec.cap;
     for (int r = threadIdx.x & 31; r < n; r += 32) {
+        int32_t* c = col + b + 4 * (int64_t)r;
+        double* x = val + b + 4 * (int64_t)r;
+        if (r >= rec.cap) {
+            for (int q = 0; q < 4; ++q) {
+                c[q] = 0;
+                x[q] = nan("");
+            }
+            continue;
+        }
         const rt_run v = row[r];
         CellAcc<float> a;
         a.W = v.w00;
@@ -1000,8 +1012,6 @@ __global__ void __launch_bounds__(kBlock) k_rows_expand(int n_pairs, int nx, con
         a.Wxy = v.w11;
         double w00, w10, w01, w11;
         a.node_weights(w00, w10, w01, w11);
-        int32_t* c = col + b + 4 * (int64_t)r;
-        double* x = val + b + 4 * (int64_t)r;
         if (vec) {
             *reinterpret_cast<int4*>(c) = make_int4(v.node, v.node + 1, v.node + nx, v.node + nx + 1);
             reinterpret_cast<double2*>(x)[0] = make_double2(w00, w10);

@@ -1,6 +1,7 @@
 """rt_path_matrix where memory is short: the matrix from one trace keeps a
 record of about the matrix's size, and a call that has room for the matrix
 alone gives the same matrix by counting and filling."""
+import ctypes as C
 import types
 import weakref
 
@@ -130,3 +131,31 @@ def test_record_belongs_to_the_stream_that_uses_it(rt, case, handle, monkeypatch
     assert empty.stream.cuda_stream == side.cuda_stream != torch.cuda.current_stream().cuda_stream
     side.synchronize()
     _same(got, want)
+
+
+@pytest.mark.parametrize("cap", [1, 8, 31, 33])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_rows_longer_than_their_record(rt, case, cap, shift):
+    """Nothing is read past a row's record: the entries beyond it are column 0 and NaN."""
+    from paper_2511_18511_gb300 import _lib as L
+    prob, theta, ds, (row_ptr, col, val) = case
+    ctx = rt.default_context(prob.c.device.index)
+    runs = torch.empty(prob.n_pairs * cap * L.RUN_BYTES, dtype=torch.uint8, device="cuda")
+    rp = torch.empty_like(row_ptr)
+    nnz = C.c_int64(0)
+    ps, o, rec = prob.struct(), rt._opts(ds), L.RtRows(runs.data_ptr(), None, cap)
+    s = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    rc = ctx.lib.rt_path_record(ctx.h, C.byref(ps), C.byref(o), C.c_void_p(theta.data_ptr()), C.byref(rec),
+                                C.c_void_p(rp.data_ptr()), C.byref(nnz), s)
+    assert rc == L.RT_ENOMEM and nnz.value == col.numel() and torch.equal(rp, row_ptr)
+    # shift 1: stores of single entries
+    c = torch.full((shift + nnz.value,), -7, dtype=torch.int32, device="cuda")[shift:]
+    v = torch.full((shift + nnz.value,), -7.0, dtype=torch.float64, device="cuda")[shift:]
+    rc = ctx.lib.rt_path_expand(ctx.h, C.byref(ps), C.byref(rec), C.c_void_p(rp.data_ptr()), C.c_void_p(c.data_ptr()),
+                                C.c_void_p(v.data_ptr()), s)
+    assert rc == L.RT_OK
+    row = torch.repeat_interleave(torch.arange(prob.n_pairs, device="cuda"), row_ptr.diff())
+    kept = torch.arange(nnz.value, device="cuda") - row_ptr[row] < 4 * cap
+    assert not bool(kept.all())
+    assert torch.equal(c, torch.where(kept, col, 0))
+    assert torch.equal(v[kept], val[kept]) and torch.isnan(v[~kept]).all()
