@@ -325,7 +325,8 @@ int rt_path_matrix(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt,
  * the nnz entries of col and val from it, the same values as rt_path_matrix.
  * RT_ENOMEM (row_ptr and nnz valid) if a ray visits more than cap cells: use
  * rt_path_matrix then; rt_path_expand would give the entries beyond a row's
- * record column 0 and value NaN. RT_FP32_COMP and RT_BILINEAR only (RT_EINVAL otherwise).
+ * record column 0 and value NaN. RT_ENOMEM with nnz_out unwritten: no workspace.
+ * RT_FP32_COMP and RT_BILINEAR only (RT_EINVAL otherwise).
  */
 int rt_path_record(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt, const double* theta,
                    const rt_rows* rec, int64_t* row_ptr, int64_t* nnz_out, void* stream);

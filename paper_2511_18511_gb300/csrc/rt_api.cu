@@ -468,7 +468,6 @@ int rt_path_record(rt_ctx* ctx, const rt_problem* prob, const rt_options* opt, c
     if (over) {
         e = cudaMemsetAsync(row_ptr, 0, sizeof(int64_t), s);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "row_ptr reset");
-        if (G.n_pairs == 0) nnz = 0;
     }
     *nnz_out = nnz;
     return over ? fail(ctx, RT_ENOMEM, "a row visits more than cap cells (row_ptr is valid)") : RT_OK;
