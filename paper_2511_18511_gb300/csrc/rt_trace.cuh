@@ -267,9 +267,15 @@ struct Cell<float> {
     __device__ __forceinline__ void load(int i, int j) {
         pi = i;
         pj = j;
-        // clamp for memory safety; rays stay inside by the ring/grid check
-        const unsigned w = (unsigned)(nx - 1);
-        const V* p = F + min((unsigned)j * w + (unsigned)i, w * (unsigned)(ny - 1) - 1u);
+        // to the edge cell on each axis, as in FP64, one instruction each:
+        // max(min(i, nx - 2), 0). The ring check leaves a step and a cell around
+        // the ring; stages of steps of several cells in a steep field go beyond.
+        // One clamp of the linear index, which took another row's cell there, was
+        // 0.2 to 0.6 % faster (63 rays of 128^2: 345 us, 347 now; 4,032 linked
+        // pairs 1.310 ms, 1.313 now).
+        i = __vimin_s32_relu(i, nx - 2);
+        j = __vimin_s32_relu(j, ny - 2);
+        const V* p = F + ((unsigned)j * (unsigned)(nx - 1) + (unsigned)i);
         asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(sa.v), "=l"(sx.v), "=l"(sy.v), "=l"(sxy.v) : "l"(p));
         asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4 + 32];" : "=l"(ga.v), "=l"(gx.v), "=l"(gy.v), "=l"(gxy.v) : "l"(p));
     }
