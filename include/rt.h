@@ -489,7 +489,7 @@ enum rtborn_gemm {
  *   prob      grid, c_mps, n_tx, tx_xy_mm, ring_radius_mm (pairs ignored).
  *   opt       precision must be RT_FP32_COMP; ds_mm in (0, h]; blocks_per_sm
  *             picks the fan kernel variant (resident 128-thread blocks per SM
- *             it is compiled for): 0 (= 6, or 5 with absorption), 4, 5, 6 or 8;
+ *             it is compiled for): 0 (= 5), 4, 5, 6 or 8;
  *             interpolator RT_BSPLINE takes c, its gradient and its Hessian
  *             from the interpolating cubic B-spline of c (analytic derivatives;
  *             the paper's choice for ray-Born, Sec. 3.3.1) and s from the spline

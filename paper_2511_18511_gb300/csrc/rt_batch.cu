@@ -174,7 +174,9 @@ __global__ void __launch_bounds__(BLOCK, MINB)
 // a retrace inside k_batch, on whichever lane had linked the pair, it shared
 // the loop with unrelated linking rays and its sink cost the link registers:
 // eight instances of up to 768^2 nodes and 256 transducers took 31.2 ms then,
-// 24.5 ms now (25.3 ms at 5 blocks an SM in place of 4, 26.6 ms at 6).
+// 24.5 ms now. Compiled for 6 blocks an SM (80 registers, 52 bytes spilled): the
+// whole call takes 24.5 ms, with 5 blocks (96 registers, no spill) 25.4, with 4
+// (102) 25.6; the chains of cell reloads want the warps more than the registers.
 template <typename T>
 __global__ void __launch_bounds__(128, LinkOcc<T>::blocks)
     k_batch_adjoint(const __grid_constant__ BatchParams P, long long total, unsigned long long* counters, int lanes) {
@@ -295,6 +297,8 @@ extern "C" int rt_batch_run(rt_ctx* ctx, int32_t n_inst, const rt_instance* inst
     if (opt->subfan_rays != 0) return rt::set_error(ctx, RT_EINVAL, "rt_batch_run links in one launch: subfan_rays must be 0");
     const int block = opt->block_threads ? opt->block_threads : 128;
     const int steps = opt->step_unroll ? opt->step_unroll : 16;
+    // 4 blocks of 128 an SM by default: eight instances 24.5 ms, 24.7 at 5, 25.5 at
+    // 6. Many instances fill more (autotune.py picks per batch).
     const int bpsm = opt->blocks_per_sm ? opt->blocks_per_sm
                                         : (opt->precision == RT_FP64 ? 1 : 512 / block);
     const size_t nb = rt::node_bytes(opt->precision);

@@ -726,7 +726,8 @@ __device__ __forceinline__ void heun_step(Cell<float>& C, const RayState<float>&
 // Each ray leaves its cell about every eighth step, and the warp then pays for
 // both forms of the step: worth it for one to three lanes (one ray 300 ns a
 // step against 348 without at the time; 1 or 6 lanes in place of 3 change the
-// cold link by less than its runs differ). One-trace kernels of wide warps
+// cold link of 261,632 pairs by less than its runs differ, which is where the line
+// was tried; launches of 4 or 5 lanes a warp were not measured). One-trace kernels of wide warps
 // leave the form out: it made the adjoint 10 % slower through its registers.
 constexpr int kSparseLanes = 3;
 __device__ __forceinline__ bool sparse_warp() { return __popc(__activemask()) <= kSparseLanes; }
