@@ -156,6 +156,12 @@ struct BornCell {
     }
 
     // Fields at fractions (u, v) of cell (ci, cj), as Cell::at of the ToF path.
+    // The move to another cell by offsets (axis_move) is the cheaper one where
+    // instructions count: RK4 maps of 24 transducers at 192^2 4.25 ms by comparisons
+    // (CMP), 4.02 by offsets. Heun's two samples a step are a short chain, which the
+    // offsets lengthen: 8 transducers at 128^2 1.67 ms by comparisons and 1.87 by
+    // offsets (with absorption 1.73 and 1.93), 32 at 256^2 4.36 and 4.25.
+    template <bool CMP = false>
     __device__ __forceinline__ void at(int ci, int cj, float u, float v, float& c, float& gx, float& gy, float& hxx,
                                        float& hxy, float& hyy, float& tx, float& ty) {
         // 0 <= u < 1 on the float bits (-0 takes the general path, to the same result)
@@ -164,12 +170,22 @@ struct BornCell {
             ty = v;
         } else {
             int i, j;
-            float ox, oy;
-            axis_move(u, ci, i, ox);
-            axis_move(v, cj, j, oy);
-            tx = u + ox;
-            ty = v + oy;
-            if (!(u >= -1.f && u < 2.f && v >= -1.f && v < 2.f)) {
+            const bool near = u >= -1.f && u < 2.f && v >= -1.f && v < 2.f;
+            if (CMP && near) {
+                const bool ul = u < 0.f, uh = u >= 1.f, vl = v < 0.f, vh = v >= 1.f;
+                tx = ul ? u + 1.f : (uh ? u - 1.f : u);
+                ty = vl ? v + 1.f : (vh ? v - 1.f : v);
+                i = ci + (ul ? -1 : (uh ? 1 : 0));
+                j = cj + (vl ? -1 : (vh ? 1 : 0));
+            }
+            if (!CMP) {
+                float ox, oy;
+                axis_move(u, ci, i, ox);
+                axis_move(v, cj, j, oy);
+                tx = u + ox;
+                ty = v + oy;
+            }
+            if (!near) {
                 const float fu = floorf(u), fv = floorf(v);
                 i = ci + (int)fu;
                 j = cj + (int)fv;
@@ -233,6 +249,7 @@ struct BornCellS {
         }
     }
 
+    template <bool CMP = false>   // one form of the move here
     __device__ __forceinline__ void at(int ci, int cj, float u, float v, float& c, float& gx, float& gy, float& hxx,
                                        float& hxy, float& hyy, float& tx, float& ty) {
         int i, j;
@@ -309,7 +326,7 @@ __device__ __forceinline__ void born_heun(CellB& C, const BornRay& B, float H, f
     float tx, ty, k1x, k1y, k1Q, k1P, k2x, k2y, k2Q, k2P;
     born_rhs(c, gx, gy, hxx, hxy, hyy, dx, dy, B.Q, B.P, k1x, k1y, k1Q, k1P);
     const float e2x = dx + H * k1x, e2y = dy + H * k1y, Q2 = B.Q + H * k1Q, P2 = B.P + H * k1P;
-    C.at(B.S.ci, B.S.cj, B.S.fx + H * dx, B.S.fy + H * dy, c, gx, gy, hxx, hxy, hyy, tx, ty);
+    C.template at<true>(B.S.ci, B.S.cj, B.S.fx + H * dx, B.S.fy + H * dy, c, gx, gy, hxx, hxy, hyy, tx, ty);
     born_rhs(c, gx, gy, hxx, hxy, hyy, e2x, e2y, Q2, P2, k2x, k2y, k2Q, k2P);
     N.Q = B.Q + Hh * (k1Q + k2Q);
     N.P = B.P + Hh * (k1P + k2P);
