@@ -196,6 +196,9 @@ int make_geom(rt_ctx* ctx, const rt_problem* p, const rt_options* o, Geom* G) {
     if (Rc * Rc > 1.0e8 || g.nx > 16384 || g.ny > 16384)
         return fail(ctx, RT_EINVAL, "ring or grid too large (at most 16384 nodes per axis)");
     G->nx = g.nx;
+    G->ilast = g.nx - 2;
+    G->jlast = g.ny - 2;
+    G->row = g.nx - 1;
     G->ny = g.ny;
     G->h = g.h_mm;
     G->x0 = g.x0_mm;

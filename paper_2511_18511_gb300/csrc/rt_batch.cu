@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(BLOCK, MINB)
     extern __shared__ unsigned char smem[];
     LinkState& L = reinterpret_cast<LinkState*>(smem)[threadIdx.x];
     Cell<T> C;
-    C.F = nullptr; C.nx = 3; C.ny = 3; C.pi = INT_MIN; C.pj = INT_MIN;
+    C.F = nullptr; C.pi = INT_MIN; C.pj = INT_MIN;
     TraceState<T> ts;
     NoSink sink;
     long long steps = 0;
@@ -83,8 +83,7 @@ __global__ void __launch_bounds__(BLOCK, MINB)
             const int k = queue_pair(G, (int)(q - d.pair_base));
             if (C.F != d.field) {
                 C.F = static_cast<const CellCoef<T>*>(d.field);
-                C.nx = G.nx;
-                C.ny = G.ny;
+                C.grid(G);
                 C.pi = INT_MIN;
                 C.pj = INT_MIN;
             }
@@ -174,7 +173,7 @@ __global__ void __launch_bounds__(BLOCK, MINB)
 // a retrace inside k_batch, on whichever lane had linked the pair, it shared
 // the loop with unrelated linking rays and its sink cost the link registers:
 // eight instances of up to 768^2 nodes and 256 transducers took 31.2 ms then,
-// 24.5 ms now. Compiled for 6 blocks an SM (80 registers, 52 bytes spilled): the
+// 24.5 ms now. Compiled for 6 blocks an SM (80 registers, 60 bytes spilled): the
 // whole call takes 24.5 ms, with 5 blocks (96 registers, no spill) 25.4, with 4
 // (102) 25.6; the chains of cell reloads want the warps more than the registers.
 template <typename T>
@@ -192,8 +191,7 @@ __global__ void __launch_bounds__(128, LinkOcc<T>::blocks)
         if (w != 0.0 && isfinite(w) && setup_pair(G, k, X)) {
             Cell<T> C;
             C.F = static_cast<const CellCoef<T>*>(d.field);
-            C.nx = G.nx;
-            C.ny = G.ny;
+            C.grid(G);
             C.pi = INT_MIN;
             C.pj = INT_MIN;
             AdjSink<T> sink;

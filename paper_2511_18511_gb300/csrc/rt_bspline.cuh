@@ -48,6 +48,8 @@ struct CellS {
     const V* pc;            // its coefficients
     T a[16];                // c: a[4q + p] multiplies tx^p ty^q
 
+    __device__ __forceinline__ void grid(const Geom& G) { nx = G.nx; ny = G.ny; }
+
     __device__ __forceinline__ void load(int i, int j) {
         pi = i;
         pj = j;

@@ -91,8 +91,7 @@ template <typename T, int I>
 __device__ __forceinline__ typename Samp<T, I>::CellT make_cell(const Geom& G, const typename Samp<T, I>::Field* F) {
     typename Samp<T, I>::CellT C;
     C.F = F;
-    C.nx = G.nx;
-    C.ny = G.ny;
+    C.grid(G);
     C.pi = INT_MIN;
     C.pj = INT_MIN;
     return C;

@@ -70,6 +70,7 @@ struct Geom {
     // FP32 copies of the per-step constants, so the FP32 march issues no FP64
     float Hf, dsf, Rcf, oxff, oyff, qf;
     double Hd, Rcd;         // ds / h and R / h
+    int ilast, jlast, row;  // nx - 2, ny - 2: the last cell of an axis; nx - 1: cells per row
     int Qi;                 // Q as 32-bit (grids up to 32k cells per side)
 };
 
@@ -212,6 +213,8 @@ struct Cell {
     T ya, ybx, yby, ybxy;             // h dc/dy
     T sa, sbx, sby, sbxy;             // s
 
+    __device__ __forceinline__ void grid(const Geom& G) { nx = G.nx; ny = G.ny; }
+
     __device__ __forceinline__ void load(int i, int j) {
         pi = i;
         pj = j;
@@ -263,10 +266,12 @@ template <>
 struct Cell<float> {
     using V = CellCoef<float>;
     const V* __restrict__ F;
-    int nx, ny;
+    int ilast, jlast, row;            // Geom's
     int pi, pj;                       // cached cell
     F2 sa, sx, sy, sxy;               // (c, s) = sa + tx sx + ty (sy + tx sxy)
     F2 ga, gx, gy, gxy;               // (h dc/dx, h dc/dy)
+
+    __device__ __forceinline__ void grid(const Geom& G) { ilast = G.ilast; jlast = G.jlast; row = G.row; }
 
     __device__ __forceinline__ void load(int i, int j) {
         pi = i;
@@ -274,12 +279,14 @@ struct Cell<float> {
         // to the edge cell on each axis, as in FP64, one instruction each:
         // max(min(i, nx - 2), 0). The ring check leaves a step and a cell around
         // the ring; stages of steps of several cells in a steep field go beyond.
-        // One clamp of the linear index, which took another row's cell there, was
-        // 0.2 to 0.6 % faster (63 rays of 128^2: 345 us, 347 now; 4,032 linked
-        // pairs 1.310 ms, 1.313 now).
-        i = __vimin_s32_relu(i, nx - 2);
-        j = __vimin_s32_relu(j, ny - 2);
-        const V* p = F + ((unsigned)j * (unsigned)(nx - 1) + (unsigned)i);
+        // The bounds come from the kernel's parameter: formed here from nx and ny
+        // they cost registers (all travel times of 261,632 pairs at 1024^2 16.7 ms
+        // against 15.1, 65,280 adjoints 5.03 against 4.95). One clamp of the linear
+        // index, which took another row's cell out there, measures the same (0.1 % on
+        // the mean of fifty calls, links, travel times, adjoints and batches).
+        i = __vimin_s32_relu(i, ilast);
+        j = __vimin_s32_relu(j, jlast);
+        const V* p = F + ((unsigned)j * (unsigned)row + (unsigned)i);
         asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(sa.v), "=l"(sx.v), "=l"(sy.v), "=l"(sxy.v) : "l"(p));
         asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4 + 32];" : "=l"(ga.v), "=l"(gx.v), "=l"(gy.v), "=l"(gxy.v) : "l"(p));
     }
