@@ -1071,11 +1071,11 @@ def _kernel_hash(files=("rt_trace.cuh", "rt_link.cuh", "rt_bspline.cuh", "rt_ray
 
 
 BORN_HASH_FILES = ("rt_trace.cuh", "rt_bspline.cuh", "rt_born.cu")
-BATCH_HASH_FILES = ("rt_trace.cuh", "rt_link.cuh", "rt_batch.cu")
+BATCH_HASH_FILES = ("rt_trace.cuh", "rt_link.cuh", "rt_ray.cu", "rt_batch.cu")
 # the k_batch variant (rays per block, RK4 steps per queue check, blocks per SM)
 # of the committed batch captures; the batch leg reports their traffic only when
 # the autotuner picked this variant
-BATCH_PROFILE_VARIANT = (128, 16, 5)
+BATCH_PROFILE_VARIANT = (128, 16, 6)
 
 
 def _traffic(path: str, files) -> "int | None":
