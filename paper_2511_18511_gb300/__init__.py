@@ -296,7 +296,8 @@ def _path_matrix_recorded(ctx, ps, o, th, row_ptr, cap: int, size: int, stream):
         # stream's pool may still be in use there, and would go back there too early
         own = stream                         # None: the current one
         if stream is not None and not isinstance(stream, torch.cuda.Stream):
-            own = torch.cuda.ExternalStream(stream.cuda_stream, device=dev)
+            h = stream.cuda_stream           # 0: ExternalStream would make a new stream
+            own = torch.cuda.ExternalStream(h, device=dev) if h else torch.cuda.default_stream(dev)
         with torch.cuda.stream(own):
             runs = torch.empty(size, dtype=torch.uint8, device=dev)
         rec = _L.RtRows(runs.data_ptr(), None, cap)

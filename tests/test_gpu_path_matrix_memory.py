@@ -159,3 +159,15 @@ def test_rows_longer_than_their_record(rt, case, cap, shift):
     assert not bool(kept.all())
     assert torch.equal(c, torch.where(kept, col, 0))
     assert torch.equal(v[kept], val[kept]) and torch.isnan(v[~kept]).all()
+
+
+def test_record_on_the_default_stream_by_its_handle(rt, case, monkeypatch):
+    prob, theta, ds, want = case
+    torch.cuda.synchronize()
+    empty = _Record()
+    monkeypatch.setattr(torch, "empty", empty)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        got = rt.rt_path_matrix(prob, theta, ds, stream=types.SimpleNamespace(cuda_stream=0))
+    assert empty.stream.cuda_stream == 0
+    torch.cuda.synchronize()
+    _same(got, want)
